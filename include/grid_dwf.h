@@ -111,7 +111,12 @@ int grid_dwf_set_stream(grid_dwf_t* h, void* stream);
  * Mpc^+ Mpc, the FP64 CG and the FP64 true residuals of the mixed CG) and of the FP64 fermion
  * force (grid_dwf_force, grid_dwf_pf_force with precision GRID_DWF_FP64); storage stays FP64, and
  * so do the vector updates and reductions of the solvers.
- * GRID_DWF_FP64_ARITH_NATIVE (the default): IEEE double. GRID_DWF_FP64_ARITH_FLOAT_FLOAT: each
+ * GRID_DWF_FP64_ARITH_NATIVE (the default): double precision. The hopping sum itself is formed in
+ * 64-bit integer blocks (a neighbour's 24 reals of one slice share the exponent of the largest; sums
+ * exact, one rounding per hop), with errors below those of IEEE arithmetic relative to the largest
+ * real of the (site, slice)'s neighbours, and in IEEE double where a magnitude lies outside
+ * 2^-400 .. 2^400 (infinities, NaN and subnormals included); everything else is IEEE double.
+ * GRID_DWF_FP64_ARITH_FLOAT_FLOAT: each
  * real carried as an unevaluated sum of two floats (Dekker's double-length arithmetic: error-free
  * TwoSum and FMA-based TwoProduct), about 46 significant bits (relative error of an operator
  * application ~1e-14) on the FP32 pipe, which on this GPU has ~64 times the FP64 pipe's

@@ -35,6 +35,7 @@ struct grid_dwf {
   size_t l2_bytes = (size_t)126 << 20;  // the device's L2 (read at create)
   double* U_canon = nullptr;            // canonical FP64 links, device
   void* gauge[4][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
+  void* gauge_fx[2] = {nullptr, nullptr};  // links as integer blocks (the FP64 hop), per parity
   std::map<int, std::pair<void*, size_t>> ws;  // workspace buffers by id
   double* partials = nullptr;           // reduction partial sums
   double* scal = nullptr;               // CG scalars (device)
@@ -195,6 +196,11 @@ int finish(grid_dwf_t* h, const char* where) {
 
 int ensure_gauge(grid_dwf_t* h, int prec) {
   if (!h->U_canon) return fail(h, GRID_DWF_ERR_NO_GAUGE, "no gauge field set (call grid_dwf_set_gauge)");
+  if (prec == GRID_DWF_FP64 && h->fp64_arith == GRID_DWF_FP64_ARITH_NATIVE && !h->gauge_fx[1]) {
+    for (auto& q : h->gauge_fx)
+      if (!q) CK(cudaMalloc(&q, (size_t)h->g.N4h * 4 * FX_LINK_BYTES), "gauge allocation");
+    CK(launch_pack_gauge_fx(h->c12, h->g, h->U_canon, h->gauge_fx[0], h->gauge_fx[1], h->stream), "pack gauge");
+  }
   if (h->gauge[prec][0]) return GRID_DWF_OK;
   const size_t lb = link_bytes(prec_bytes(prec), h->c12);
   const size_t bytes = (size_t)h->g.N4h * 4 * lb;
@@ -300,7 +306,10 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
       a.div_lt = make_fastdiv((uint32_t)h->g.L[3]);
     }
   }
+  a.Ufx_out = h->gauge_fx[out_parity];
+  a.Ufx_in = h->gauge_fx[1 - out_parity];
   a.alpha = alpha;
+  a.alpha_log2 = std::ilogb(alpha);
   a.beta = beta;
   a.d5 = h->d5;
   a.mass = h->mass;
@@ -308,17 +317,21 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
   a.inv_den = h->inv_den;
   int threads = a.nsg * a.sites_per_cta;
   int blocks = (h->g.N4h + a.sites_per_cta - 1) / a.sites_per_cta;
-  const size_t rbytes = prec == GRID_DWF_FP64 ? 8 : 4;
-  size_t smem = dhop_link_smem_bytes(prec, a.sites_per_cta, h->c12) +
-                (post == POST_NONE                ? 0
-                 : prec == GRID_DWF_FP64 ? (size_t)a.sites_per_cta * h->Ls * INV_SLICE_STRIDE * rbytes
-                                         : (size_t)a.sites_per_cta * inv_site_stride(h->Ls) * rbytes);
+  size_t smem = dhop_link_smem_bytes(a.sites_per_cta) +
+                (post == POST_NONE ? 0 : (size_t)a.sites_per_cta * inv_site_stride(h->Ls) * sizeof(float));
   cudaError_t e;
   if (prec == GRID_DWF_FP64 && h->fp64_arith == GRID_DWF_FP64_ARITH_FLOAT_FLOAT) {
     smem = dhop_ff_smem_bytes(a.sites_per_cta, h->Ls, post != POST_NONE);
     e = launch_dhop_ff(a, dag, h->c12, threads, blocks, smem, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "dhop launch (float-float)");
     return GRID_DWF_OK;
+  }
+  if (prec == GRID_DWF_FP64) {
+    // two threads per slice: half as many sites fill a CTA
+    a.sites_per_cta = std::max(1, a.sites_per_cta / 2);
+    threads = 2 * a.nsg * a.sites_per_cta;
+    blocks = (h->g.N4h + a.sites_per_cta - 1) / a.sites_per_cta;
+    smem = dhop_fx_smem_bytes(a.sites_per_cta, h->Ls, post != POST_NONE);
   }
   switch (prec) {
     case GRID_DWF_FP64: e = launch_dhop<P64>(a, dag, h->c12, threads, blocks, smem, h->stream); break;
@@ -331,11 +344,11 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
 }
 
 // Both halves of a full-lattice hop (each output half from the other input half, independent):
-// one launch for the packed precisions (one ramp-up and tail instead of two), two for FP64.
+// one launch (one ramp-up and tail instead of two), two for FP64 in float-float arithmetic.
 int dhop_full(grid_dwf_t* h, int prec, const char* in, char* out, bool dag, int pre, double alpha, double beta,
               const char* aux, const CgEpilogue& epi = CgEpilogue()) {
   const size_t hb = half_bytes(h, prec);
-  if (prec == GRID_DWF_FP64) {
+  if (prec == GRID_DWF_FP64 && h->fp64_arith == GRID_DWF_FP64_ARITH_FLOAT_FLOAT) {
     RET(dhop_half(h, prec, in + hb, out, 0, dag, pre, POST_NONE, alpha, beta, aux));
     return dhop_half(h, prec, in, out + hb, 1, dag, pre, POST_NONE, alpha, beta, aux ? aux + hb : nullptr);
   }
@@ -496,6 +509,7 @@ int grid_dwf_destroy(grid_dwf_t* h) {
   cudaFree(h->U_canon);
   for (auto& pp : h->gauge)
     for (auto& q : pp) cudaFree(q);
+  for (auto& q : h->gauge_fx) cudaFree(q);
   for (auto& kv : h->ws) cudaFree(kv.second.first);
   cudaFree(h->partials);
   cudaFree(h->scal);
@@ -532,6 +546,8 @@ int grid_dwf_set_gauge(grid_dwf_t* h, const double* U) {
   CK(cudaMemcpyAsync(h->U_canon, U, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->stream),
      "gauge copy");
   if (!on_device) CK(cudaStreamSynchronize(h->stream), "gauge copy");
+  if (h->gauge_fx[1])
+    CK(launch_pack_gauge_fx(h->c12, h->g, h->U_canon, h->gauge_fx[0], h->gauge_fx[1], h->stream), "pack gauge");
   for (int p = 0; p < 4; ++p)
     if (h->gauge[p][0]) CK(launch_pack_gauge(p, h->c12, h->g, h->U_canon, h->gauge[p][0], h->gauge[p][1], h->stream), "pack gauge");
   return finish(h, "set_gauge");

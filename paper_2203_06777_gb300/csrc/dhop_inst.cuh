@@ -1,5 +1,5 @@
-// Instantiates launch_dhop<DWF_PREC>: one translation unit per storage precision so that the
-// kernel variants of the four precisions compile in parallel.
+// Instantiates launch_dhop<DWF_PREC> of a packed precision (FP32, FP16, BF16): one translation
+// unit per precision so that the kernel variants compile in parallel.
 #include "dhop_kernel.cuh"
 
 namespace gdwf {
@@ -15,9 +15,7 @@ static cudaError_t launch_one(const DhopArgs& a, int threads, int blocks, size_t
       configured = smem;
     }
   }
-  if constexpr (DWF_PREC == P64) {
-    kern<<<blocks, threads, smem, stream>>>(a);
-  } else {
+  {
     // full CTAs only (the packed kernel has no tail handling); a ragged end gets one more CTA (per
     // half) flush with the end of the lattice, launched after the first so no two writes overlap
     // in time. a.in2 != nullptr: both halves of a full-lattice hop in the same launches.
@@ -63,12 +61,7 @@ static cudaError_t launch_one(const DhopArgs& a, int threads, int blocks, size_t
 template <int LSC>
 static cudaError_t launch_ls(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
                              cudaStream_t stream) {
-  if constexpr (DWF_PREC == P64) {
-    if (dag) return c12 ? launch_one<true, true, LSC, EPI_BOTH>(a, threads, blocks, smem, stream)
-                        : launch_one<true, false, LSC, EPI_BOTH>(a, threads, blocks, smem, stream);
-    return c12 ? launch_one<false, true, LSC, EPI_BOTH>(a, threads, blocks, smem, stream)
-               : launch_one<false, false, LSC, EPI_BOTH>(a, threads, blocks, smem, stream);
-  } else {
+  {
     // the instantiation with exactly the epilogue parts this launch uses; the CG epilogues exist
     // for the launches that use them only: Mpc's second launch (pre-operation Mooee, no dag) with
     // the norm, Mpc^+'s second launch (Mooee^+, dag) with the update, 18-real links

@@ -15,8 +15,8 @@
 // Thread mapping. FP32 and the 16-bit storage formats: one thread per (4D checkerboard site,
 // slice pair); every real of the two slices is a float2 and each hop (projection, SU(3)
 // product, reconstruction) runs on packed two-wide FP32 instructions, one instruction for two
-// slices. FP64: one thread per (site, slice) with scalar arithmetic (the FP64 pipe, not the
-// instruction issue, bounds it). All threads of a site load the same link (a broadcast load), so
+// slices. FP64 has a kernel of its own (dhop_p64.cu), which shares the arguments, the layout and
+// the epilogues. All threads of a site load the same link (a broadcast load), so
 // every link is read from memory once per site and reused for all Ls slices; a CTA holds whole
 // sites, which the fused Mooee^-1 epilogue needs.
 //
@@ -86,6 +86,11 @@ struct DhopArgs {
   // Full-lattice launches: 1 to alternate the CTAs between the two halves (CTA 2b + h: CTA b of
   // half h) instead of running all CTAs of the first half first.
   int interleave;
+  // FP64 kernel (dhop_p64.cu): the links as integer blocks, output and input parity, and log2 |alpha|
+  // (alpha is a signed power of two in every launch)
+  const void* Ufx_out;
+  const void* Ufx_in;
+  int alpha_log2;
   double alpha, beta;
   double d5;       // 5 - M5
   double mass;     // m
@@ -250,44 +255,18 @@ __device__ __forceinline__ void load_link(const char* p, typename Store<P>::R* u
   if (C12) reconstruct_row2(u);
 }
 
-// A link from shared memory (plain loads; the staged kernel reads its own buffers).
-template <int P, bool C12>
-__device__ __forceinline__ void load_link_smem(const char* p, typename Store<P>::R* u) {
-  using R = typename Store<P>::R;
-  constexpr int VEC = Store<P>::VEC;
-  constexpr int NR = C12 ? 12 : 18;
-  constexpr int NV = (NR + VEC - 1) / VEC;
-  R buf[NV * VEC];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) ld16c<P>(p + v * 16, buf + v * VEC);
-#pragma unroll
-  for (int i = 0; i < NR; ++i) u[i] = buf[i];
-  if (C12) reconstruct_row2(u);
-}
-
-// Copy one stored link (whole 16-byte vectors) from global to shared memory.
-template <int P, bool C12>
-__device__ __forceinline__ void copy_link(char* dst, const char* src) {
-  constexpr int LB = link_bytes(sizeof(typename Store<P>::T), C12);
-#pragma unroll
-  for (int v = 0; v < LB / 16; ++v)
-    *reinterpret_cast<uint4*>(dst + v * 16) = __ldg(reinterpret_cast<const uint4*>(src + v * 16));
-}
-
-// The direct kernel stages each site's eight links in shared memory once per CTA; every slice
-// pair of the site then reads them from there. FP64 keeps the stored format (18 or 12 doubles per
-// link). The packed kernels keep every link as 18 FP32 reals (80 bytes, converted from 16-bit
-// storage and with the third row rebuilt once per site instead of once per thread), and pad each
-// site's 640 bytes by 16: the four sites that one warp reads from then start 16 bytes apart
-// modulo 128 and their 16-byte reads fall in different banks instead of four-way conflicts.
+// The packed kernels stage each site's eight links in shared memory once per CTA; every slice
+// pair of the site then reads them from there. Every link is kept as 18 FP32 reals (80 bytes,
+// converted from 16-bit storage and with the third row rebuilt once per site instead of once per
+// thread), and each site's 640 bytes are padded by 16: the four sites that one warp reads from then
+// start 16 bytes apart modulo 128 and their 16-byte reads fall in different banks instead of
+// four-way conflicts.
 constexpr int DHOP_LINK_F32_BYTES = 80;
-__host__ __device__ constexpr int dhop_link_site_bytes(int prec, bool c12) {
-  return prec == P64 ? 8 * link_bytes(8, c12) : 8 * DHOP_LINK_F32_BYTES + 16;
-}
+constexpr int DHOP_LINK_SITE_BYTES = 8 * DHOP_LINK_F32_BYTES + 16;
 
 // Shared memory of the staged links of one CTA, a multiple of 16 bytes.
-__host__ __device__ constexpr size_t dhop_link_smem_bytes(int prec, int sites_per_cta, bool c12) {
-  return (size_t)sites_per_cta * dhop_link_site_bytes(prec, c12);
+__host__ __device__ constexpr size_t dhop_link_smem_bytes(int sites_per_cta) {
+  return (size_t)sites_per_cta * DHOP_LINK_SITE_BYTES;
 }
 
 // One link from global memory (any storage precision, 18 or 12 reals) to shared memory as 18
@@ -601,28 +580,6 @@ __device__ __forceinline__ void store_lane64(char* blk, int s, int Lsh_rt, const
   for (int k = 0; k < 24; ++k) *reinterpret_cast<double*>(b + k * chunk_stride(Lsh)) = v[k];
 }
 
-// Any precision: the 24 reals of slice s (the lane of its pair), in the arithmetic type.
-template <int P, bool GLOBAL = true>
-__device__ __forceinline__ void load_slice(const char* blk, int s, int Lsh, typename Store<P>::R* v) {
-  if constexpr (P == P64) {
-    load_lane64<0, GLOBAL>(blk, s, Lsh, v);
-  } else {
-    constexpr int VEC = Store<P>::VEC, RV = Store<P>::RV, NCH = Store<P>::NCH;
-    const int l = s & 1;
-    const char* b = blk + (size_t)(s >> 1) * 16;
-#pragma unroll
-    for (int k = 0; k < NCH; ++k) {
-      float t[VEC];
-      if (GLOBAL)
-        ld16<P>(b + k * chunk_stride(Lsh), t);
-      else
-        ld16c<P>(b + k * chunk_stride(Lsh), t);
-#pragma unroll
-      for (int j = 0; j < RV; ++j) v[RV * k + j] = t[2 * j + l];
-    }
-  }
-}
-
 // Packed precisions: reals r0 .. r0 + 11 (r0 = 0: the upper, P+ spins; 12: the lower) of slice s,
 // widened to FP32.
 template <int P>
@@ -637,33 +594,6 @@ __device__ __forceinline__ void load_slice_half(const char* blk, int s, int Lsh,
 #pragma unroll
     for (int j = 0; j < RV; ++j) v[RV * k + j] = t[2 * j + l];
   }
-}
-
-// (Mooee aux)_s or (Mooee^+ aux)_s for one slice s < Ls (zero for the pad slice): the upper (P+)
-// reals couple to s-1 and the lower (P-) reals to s+1, with +m replacing -1 on the wrap-around;
-// the adjoint swaps them. GLOBAL = false reads a block staged in shared memory.
-template <int P, bool DAG5, bool GLOBAL = true>
-__device__ __forceinline__ void mooee_slice(const char* blk, int s, int Ls, int Lsh, double d5, double mass,
-                                            typename Store<P>::R* o) {
-  using R = typename Store<P>::R;
-  if (s >= Ls) {
-#pragma unroll
-    for (int r = 0; r < 24; ++r) o[r] = 0;
-    return;
-  }
-  const int sm = s > 0 ? s - 1 : Ls - 1;
-  const int sp = s < Ls - 1 ? s + 1 : 0;
-  const R cm = s > 0 ? R(-1) : R(mass);
-  const R cp = s < Ls - 1 ? R(-1) : R(mass);
-  const int s_up = DAG5 ? sp : sm, s_lo = DAG5 ? sm : sp;
-  const R c_up = DAG5 ? cp : cm, c_lo = DAG5 ? cm : cp;
-  const R d = R(d5);
-  R self[24], up[24], lo[24];
-  load_slice<P, GLOBAL>(blk, s, Lsh, self);
-  load_slice<P, GLOBAL>(blk, s_up, Lsh, up);
-  load_slice<P, GLOBAL>(blk, s_lo, Lsh, lo);
-#pragma unroll
-  for (int r = 0; r < 24; ++r) o[r] = d * self[r] + (r < 12 ? c_up * up[r] : c_lo * lo[r]);
 }
 
 // Shared-memory staging of the fifth-dimension inverse: the 24 reals of a slice, then the next
@@ -836,7 +766,7 @@ __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
   // The eight links of each site, staged once per CTA as FP32: thread q of a site fetches the
   // links of hops q, q + Lsh, ... (hop h = 2 mu + backward), so every link is requested from
   // memory once instead of once per slice pair; the hops then read them from shared memory.
-  constexpr int LSS = dhop_link_site_bytes(P, false);
+  constexpr int LSS = DHOP_LINK_SITE_BYTES;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   char* lsm = reinterpret_cast<char*>(smem_raw) + (size_t)site_local * LSS;  // [hop 8][80 bytes]
   const char* Uo = static_cast<const char*>(second ? a.Uin : a.Uout);  // links of the output parity
@@ -1010,7 +940,7 @@ __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
   // Fifth-dimension inverse through shared memory (after the staged links): whole sites live in
   // this CTA, staged as lines (inv_site_stride / inv_line_stride; the pad slice of an odd Ls is
   // stored past the line's end and never read).
-  float* sm = reinterpret_cast<float*>(smem_raw + dhop_link_smem_bytes(P, a.sites_per_cta, false));
+  float* sm = reinterpret_cast<float*>(smem_raw + dhop_link_smem_bytes(a.sites_per_cta));
   const int lst = inv_line_stride(Ls), sst = inv_site_stride(Ls);
   if (active) {
     float* d0 = sm + (size_t)site_local * sst + 2 * q;
@@ -1042,139 +972,17 @@ __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
   }
 }
 
-// FP64: one thread per (site, slice), scalar arithmetic.
-template <bool DAG, bool C12, int LSC>
-__device__ __forceinline__ void dhop_body_lane64(const DhopArgs& a) {
-  constexpr int LB = link_bytes(8, C12);
-  constexpr int SF = DAG ? +1 : -1;
-  constexpr int SB = -SF;
-  constexpr int LSHC = LSC > 0 ? ls_half(LSC) : 0;
-  const int Ls = LSC > 0 ? LSC : a.g.Ls;
-  const int Lsh = LSC > 0 ? LSHC : ls_half(a.g.Ls);
-  const int Lsp = 2 * Lsh;
-  const int tid = threadIdx.x;
-  const int site_local = tid / Lsp;
-  const int s = tid - site_local * Lsp;
-  const int site = blockIdx.x * a.sites_per_cta + site_local;
-  const bool active = site_local < a.sites_per_cta && site < a.g.N4h;
-  const size_t site_bytes = (size_t)Lsp * 24 * 8;
-  const double alpha = a.alpha;
-
-  double acc[24];
-#pragma unroll
-  for (int r = 0; r < 24; ++r) acc[r] = 0;
-  // links staged once per CTA, as in dhop_body_pair
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  char* lsm = reinterpret_cast<char*>(smem_raw);  // [site_local][hop 8][LB]
-  int c[4];
-  if (active) {
-    cb_coords(a.g, site, a.out_parity, c);
-    const char* Uo = static_cast<const char*>(a.Uout);
-    const char* Ui = static_cast<const char*>(a.Uin);
-    for (int h = s; h < 8; h += Lsp) {
-      const int mu = h >> 1;
-      const char* src;
-      if ((h & 1) == 0) {
-        src = Uo + ((size_t)site * 4 + mu) * LB;
-      } else {
-        int ph;
-        src = Ui + ((size_t)cb_neighbour(a.g, site, c, mu, false, ph) * 4 + mu) * LB;
-      }
-      copy_link<P64, C12>(lsm + ((size_t)site_local * 8 + h) * LB, src);
-    }
-  }
-  __syncthreads();
-  if (active) {
-    const char* in = static_cast<const char*>(a.in);
-#pragma unroll
-    for (int mu = 0; mu < 4; ++mu) {
-      {
-        int ph;
-        const int j = cb_neighbour(a.g, site, c, mu, true, ph);
-        double u[18], psi[24], h[12], uh[12];
-        load_link_smem<P64, C12>(lsm + ((size_t)site_local * 8 + 2 * mu) * LB, u);
-        load_lane64<LSHC>(in + site_offset(j, Lsh, site_bytes), s, Lsh, psi);
-        project<SF>(mu, psi, h);
-        su3_mul<false>(u, h, uh);
-        accumulate<SF>(mu, uh, ph < 0 ? -alpha : alpha, acc);
-      }
-      {
-        int ph;
-        const int j = cb_neighbour(a.g, site, c, mu, false, ph);
-        double u[18], psi[24], h[12], uh[12];
-        load_link_smem<P64, C12>(lsm + ((size_t)site_local * 8 + 2 * mu + 1) * LB, u);
-        load_lane64<LSHC>(in + site_offset(j, Lsh, site_bytes), s, Lsh, psi);
-        project<SB>(mu, psi, h);
-        su3_mul<true>(u, h, uh);
-        accumulate<SB>(mu, uh, ph < 0 ? -alpha : alpha, acc);
-      }
-    }
-  }
-  char* outb = static_cast<char*>(a.out) + site_offset(site, Lsh, site_bytes);
-  if (active && a.pre != PRE_NONE) {
-    const char* auxb = static_cast<const char*>(a.aux) + site_offset(site, Lsh, site_bytes);
-    double o[24];
-    if (a.pre == PRE_AUX)
-      load_lane64<LSHC>(auxb, s, Lsh, o);
-    else if (a.pre == PRE_MOOEE)
-      mooee_slice<P64, false>(auxb, s, Ls, Lsh, a.d5, a.mass, o);
-    else
-      mooee_slice<P64, true>(auxb, s, Ls, Lsh, a.d5, a.mass, o);
-#pragma unroll
-    for (int r = 0; r < 24; ++r) acc[r] = fma(a.beta, o[r], acc[r]);
-  }
-  const bool pad = s >= Ls;
-  if (a.post == POST_NONE) {
-    if (active) {
-      if (pad) {
-#pragma unroll
-        for (int r = 0; r < 24; ++r) acc[r] = 0;
-      }
-      store_lane64<LSHC>(outb, s, Lsh, acc);
-    }
-    return;
-  }
-  double* sm = reinterpret_cast<double*>(smem_raw + dhop_link_smem_bytes(P64, a.sites_per_cta, C12));
-  if (active && !pad) {
-    double* dst = sm + ((size_t)site_local * Ls + s) * INV_SLICE_STRIDE;
-#pragma unroll
-    for (int r = 0; r < 24; ++r) dst[r] = acc[r];
-  }
-  __syncthreads();
-  const int first_site = blockIdx.x * a.sites_per_cta;
-  const int nsites = min(a.sites_per_cta, a.g.N4h - first_site);
-  for (int task = tid; task < nsites * 24; task += blockDim.x) {
-    const int sl = task / 24;
-    const int r = task - sl * 24;
-    const bool upper = r < 12;
-    const bool forward_form = (a.post == POST_INV) ? upper : !upper;
-    mooee_inv_line<double>(sm + (size_t)sl * Ls * INV_SLICE_STRIDE + r, Ls, forward_form, a.mass, a.inv_d5,
-                           a.inv_den);
-  }
-  __syncthreads();
-  if (active) {
-    if (!pad) {
-      const double* src = sm + ((size_t)site_local * Ls + s) * INV_SLICE_STRIDE;
-#pragma unroll
-      for (int r = 0; r < 24; ++r) acc[r] = src[r];
-    } else {
-#pragma unroll
-      for (int r = 0; r < 24; ++r) acc[r] = 0;
-    }
-    store_lane64<LSHC>(outb, s, Lsh, acc);
-  }
-}
-
 // Register budget. Every launch of dhop_kernel has at most 128 threads (128 / threads-per-site
-// whole sites). The packed kernels keep four such CTAs per SM (128 registers per thread, no
-// spills; measured against three CTAs with 156-168 registers: FP16 storage 43.1 -> 41.0 us at
-// 16^4 x 16 and 633 -> 586 us at 32^4 x 16, FP32 and BF16 within 1-2%); the FP64 kernel is
-// bound by the FP64 pipe and keeps more registers instead.
-template <int P>
-struct DhopOccupancy {
-  static constexpr int THREADS = 128;
-  static constexpr int MIN_BLOCKS = (P == P64) ? 1 : 4;
-};
+// whole sites) and keeps four such CTAs per SM (128 registers per thread, no spills; measured
+// against three CTAs with 156-168 registers: FP16 storage 43.1 -> 41.0 us at 16^4 x 16 and 633 ->
+// 586 us at 32^4 x 16, FP32 and BF16 within 1-2%).
+constexpr int DHOP_THREADS = 128, DHOP_MIN_BLOCKS = 4;
+
+// Bytes of one link in the FP64 kernel's integer form: 9 complex entries of four words and the
+// block exponent, padded to 16 bytes.
+constexpr int FX_LINK_BYTES = 160;
+size_t dhop_fx_smem_bytes(int sites_per_cta, int Ls, bool post);
+cudaError_t launch_pack_gauge_fx(bool c12, const Geom& g, const double* canon, void* Ue, void* Uo, cudaStream_t st);
 
 // Threads per site: slice pairs (packed kernels) or padded slices (FP64).
 inline int dhop_threads_per_site(int prec, int Ls) { return prec == P64 ? ls_padded(Ls) : ls_half(Ls); }
@@ -1183,13 +991,10 @@ inline int dhop_threads_per_site(int prec, int Ls) { return prec == P64 ? ls_pad
 #define DWF_LS_SPECIALISATIONS(M) M(8) M(12) M(16)
 inline bool dhop_ls_specialised(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 
-// C12 selects the stored link format; EK the epilogue kind (EPI_BOTH for FP64).
+// C12 selects the stored link format; EK the epilogue kind.
 template <int P, bool DAG, bool C12, int LSC, int EK>
-__global__ void __launch_bounds__(DhopOccupancy<P>::THREADS, DhopOccupancy<P>::MIN_BLOCKS) dhop_kernel(const __grid_constant__ DhopArgs a) {
-  if constexpr (P == P64)
-    dhop_body_lane64<DAG, C12, LSC>(a);
-  else
-    dhop_body_pair<P, DAG, C12, LSC, EK>(a);
+__global__ void __launch_bounds__(DHOP_THREADS, DHOP_MIN_BLOCKS) dhop_kernel(const __grid_constant__ DhopArgs a) {
+  dhop_body_pair<P, DAG, C12, LSC, EK>(a);
 }
 
 // Host-side launcher, instantiated once per storage precision in its own translation unit.

@@ -25,7 +25,7 @@ from . import _build
 FP64, FP32, FP16, BF16 = 0, 1, 2, 3
 EVEN, ODD, FULL = 0, 1, 2
 CG_FP64, CG_MIXED_FP32, CG_MIXED_FP16, CG_MIXED_BF16 = 0, 1, 2, 3
-# arithmetic of the FP64 hopping term: IEEE double, or float-float (pairs of FP32 numbers)
+# arithmetic of the FP64 hopping term: double precision, or float-float (pairs of FP32 numbers)
 FP64_ARITH_NATIVE, FP64_ARITH_FLOAT_FLOAT = 0, 1
 
 STATUS = {
@@ -229,7 +229,7 @@ class GridDWF:
 
     def set_fp64_arith(self, mode: int):
         """Arithmetic of every FP64 hopping-term application on this handle (grid_dwf_set_fp64_arith):
-        FP64_ARITH_NATIVE (IEEE double) or FP64_ARITH_FLOAT_FLOAT (float-float, ~46 bits)."""
+        FP64_ARITH_NATIVE (double precision) or FP64_ARITH_FLOAT_FLOAT (float-float, ~46 bits)."""
         rc = self.lib.grid_dwf_set_fp64_arith(self._h, int(mode))
         if rc != 0:
             raise GridDWFError(rc, f"grid_dwf_set_fp64_arith: {self.lib.grid_dwf_last_error(self._h).decode()}")
