@@ -64,8 +64,8 @@ def pipe_peaks(dwf):
     return out
 
 
-KERNEL_SOURCES = ["paper_2203_06777_gb300/csrc/dhop_kernel.cuh", "paper_2203_06777_gb300/csrc/dhop_inst.cuh",
-                  "paper_2203_06777_gb300/csrc/dwf_common.cuh", "paper_2203_06777_gb300/csrc/dhop_p32.cu"]
+KERNEL_SOURCES = ["paper_2203_06777_gb300/csrc/dhop_kernel.cuh", "paper_2203_06777_gb300/csrc/dhop_packed.cu",
+                  "paper_2203_06777_gb300/csrc/dwf_common.cuh"]
 TRAFFIC_PROFILE = "profiles/dhop_fp32_16x16x16x16_ls16.md"
 TRAFFIC_PROFILE_32 = "profiles/dhop_fp32_32x32x32x32_ls16.md"
 

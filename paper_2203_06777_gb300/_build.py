@@ -1,13 +1,16 @@
 """Build libgrid_dwf.so in-tree with nvcc for sm_103a (GB300).
 
-Each translation unit under csrc/ is compiled in its own nvcc process, in parallel, then linked
-into ``paper_2203_06777_gb300/lib/libgrid_dwf.so`` with a shared CUDA runtime. A rebuild happens
-only when a source or header is newer than the library.
+Each translation unit under csrc/ is compiled in its own nvcc process (``dhop_packed.cu`` once per
+storage precision and number of slice pairs), in parallel, then linked into
+``paper_2203_06777_gb300/lib/libgrid_dwf.so`` with a shared CUDA runtime. A rebuild happens only when a
+source or header is newer than the library.
 """
 from __future__ import annotations
 
+import concurrent.futures
 import glob
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -34,6 +37,22 @@ def _sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _units():
+    """(source, object name, extra flags) of every translation unit, the slowest first."""
+    with open(os.path.join(CSRC, "dhop_kernel.cuh")) as f:
+        pairs = re.search(r"#define DWF_PAIR_SPECIALISATIONS\(M\)(.*)", f.read()).group(1)
+    units = []
+    for src in _sources():
+        name = os.path.basename(src)[:-3]
+        if name != "dhop_packed":
+            units.append((src, name, []))
+            continue
+        for n in ["0"] + re.findall(r"M\((\d+)\)", pairs):
+            for prec in ("P32", "P16", "PB16"):
+                units.insert(0, (src, f"{name}_{prec}_{n}", [f"-DDWF_PREC={prec}", f"-DDWF_PAIRS={n}"]))
+    return units
+
+
 def _deps():
     return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + [os.path.join(ROOT, "include", "grid_dwf.h"),
                                                                    os.path.abspath(__file__)]
@@ -53,22 +72,23 @@ def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = nvcc_path()
     os.makedirs(BUILD, exist_ok=True)
     os.makedirs(LIBDIR, exist_ok=True)
-    procs = []
-    objs = []
-    for src in _sources():
-        obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
-        objs.append(obj)
-        cmd = [nvcc] + NVCC_FLAGS + ["-c", src, "-o", obj]
+
+    def compile_unit(unit):
+        src, name, flags = unit
+        obj = os.path.join(BUILD, name + ".o")
+        cmd = [nvcc] + NVCC_FLAGS + flags + ["-c", src, "-o", obj]
         if verbose:
             print(" ".join(cmd), file=sys.stderr)
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
-    errors = []
-    for src, p in procs:
-        out, _ = p.communicate()
-        if p.returncode != 0:
-            errors.append(f"{os.path.basename(src)}:\n{out.decode(errors='replace')}")
-        elif verbose and out:
-            print(out.decode(errors="replace"), file=sys.stderr)
+        r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+        out = r.stdout.decode(errors="replace")
+        if verbose and out:
+            print(out, file=sys.stderr)
+        return obj, f"{name}:\n{out}" if r.returncode != 0 else None
+
+    with concurrent.futures.ThreadPoolExecutor(os.cpu_count() or 4) as pool:
+        done = list(pool.map(compile_unit, _units()))
+    objs = [obj for obj, _ in done]
+    errors = [e for _, e in done if e]
     if errors:
         raise RuntimeError("nvcc failed:\n" + "\n".join(errors))
     tmp = LIB + f".tmp{os.getpid()}"

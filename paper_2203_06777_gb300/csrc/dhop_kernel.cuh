@@ -631,6 +631,48 @@ __device__ __forceinline__ void mooee_inv_line(R* v, int Ls, bool forward_form, 
   }
 }
 
+// mooee_inv_line for FP64 with one FMA per recurrence step (v inv_d is formed once and used by both
+// sweeps): 3 FP64 instructions per value instead of 4. LS > 0: the line in registers.
+template <int LS>
+__device__ __forceinline__ void mooee_inv_line64(double* v, int Ls_rt, bool forward_form, double mass, double inv_d,
+                                                 double inv_den) {
+  constexpr int S = INV_SLICE_STRIDE;
+  const int Ls = LS > 0 ? LS : Ls_rt;
+  // the mirror form is the forward form on the reversed line
+  double* base = forward_form ? v : v + (Ls - 1) * S;
+  const int st = forward_form ? S : -S;
+  if constexpr (LS > 0) {
+    double w[LS];
+    const double v0 = base[0];
+    double acc = 0;
+#pragma unroll
+    for (int k = 1; k < LS; ++k) {
+      w[k] = base[k * st] * inv_d;
+      acc = fma(acc, inv_d, w[k]);
+    }
+    double y = fma(-mass, acc, v0) * inv_den;
+    base[0] = y;
+#pragma unroll
+    for (int k = 1; k < LS; ++k) {
+      y = fma(y, inv_d, w[k]);
+      base[k * st] = y;
+    }
+  } else {
+    double acc = 0;
+    for (int k = 1; k < Ls; ++k) {
+      const double w = base[k * st] * inv_d;
+      base[k * st] = w;
+      acc = fma(acc, inv_d, w);
+    }
+    double y = fma(-mass, acc, base[0]) * inv_den;
+    base[0] = y;
+    for (int k = 1; k < Ls; ++k) {
+      y = fma(y, inv_d, base[k * st]);
+      base[k * st] = y;
+    }
+  }
+}
+
 // The packed kernels stage the inverse differently: per site 24 lines, one per real component,
 // each holding the site's slices contiguously, so that a thread stores its two slices of a real
 // as one float2 and a line moves with 128-bit accesses. A line is padded to an odd number of
@@ -723,15 +765,14 @@ __device__ __forceinline__ void cta_sum_to(double v, double* dst) {
 }
 
 // FP32 / FP16 / BF16: one thread per (site, slice pair), packed two-wide arithmetic.
-template <int P, bool DAG, bool C12, int LSC, int EK>
+template <int P, bool DAG, bool C12, int LSHC, int EK>
 __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
   using T = typename Store<P>::T;
   constexpr int LB = link_bytes(sizeof(T), C12);
   constexpr int SF = DAG ? +1 : -1;  // forward projector (1 + SF gamma)
   constexpr int SB = -SF;            // backward projector
-  constexpr int LSHC = LSC > 0 ? ls_half(LSC) : 0;
-  const int Ls = LSC > 0 ? LSC : a.g.Ls;
-  const int Lsh = LSC > 0 ? LSHC : ls_half(a.g.Ls);
+  const int Ls = LSHC > 0 ? 2 * LSHC : a.g.Ls;
+  const int Lsh = LSHC > 0 ? LSHC : ls_half(a.g.Ls);
   const int tid = threadIdx.x;
   const int site_local = tid / Lsh;
   const int q = tid - site_local * Lsh;
@@ -955,8 +996,8 @@ __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
     const bool upper = r < 12;
     const bool forward_form = (a.post == POST_INV) ? upper : !upper;
     float* line = sm + (size_t)sl * sst + r * lst;
-    if constexpr (LSC > 0)
-      mooee_inv_line_vec<LSC>(line, forward_form, (float)a.mass, (float)a.inv_d5, (float)a.inv_den);
+    if constexpr (LSHC > 0)
+      mooee_inv_line_vec<2 * LSHC>(line, forward_form, (float)a.mass, (float)a.inv_d5, (float)a.inv_den);
     else
       mooee_inv_line<float, 1>(line, Ls, forward_form, (float)a.mass, (float)a.inv_d5, (float)a.inv_den);
   }
@@ -987,17 +1028,40 @@ cudaError_t launch_pack_gauge_fx(bool c12, const Geom& g, const double* canon, v
 // Threads per site: slice pairs (packed kernels) or padded slices (FP64).
 inline int dhop_threads_per_site(int prec, int Ls) { return prec == P64 ? ls_padded(Ls) : ls_half(Ls); }
 
-// Ls values with a compile-time specialisation; any other Ls runs the generic kernel (LSC = 0).
+// FP64 kernels: Ls values with a compile-time specialisation; any other Ls runs the generic kernel (LSC = 0).
 #define DWF_LS_SPECIALISATIONS(M) M(8) M(12) M(16)
 inline bool dhop_ls_specialised(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 
-// C12 selects the stored link format; EK the epilogue kind.
-template <int P, bool DAG, bool C12, int LSC, int EK>
+// C12 selects the stored link format; LSHC = Ls / 2 for the extents compiled in, 0 for any; EK the epilogue kind.
+template <int P, bool DAG, bool C12, int LSHC, int EK>
 __global__ void __launch_bounds__(DHOP_THREADS, DHOP_MIN_BLOCKS) dhop_kernel(const __grid_constant__ DhopArgs a) {
-  dhop_body_pair<P, DAG, C12, LSC, EK>(a);
+  dhop_body_pair<P, DAG, C12, LSHC, EK>(a);
 }
 
 // Host-side launcher, instantiated once per storage precision in its own translation unit.
+// Packed kernels: even Ls from 4 to 24 and 32 known at compile time, as pairs (the offsets of a vector's
+// chunks become immediates, the pad slice's code goes, and the inverse's lines stay in registers);
+// any other Ls runs the generic kernel. Full-lattice hop at 16^4, generic and specialised, FP32
+// Ls = 10 / 14 / 20 / 24: 57.5 / 69.7 / 82.2 / 84.3 and 47.7 / 59.9 / 75.8 / 80.5 us; FP16 Ls = 10 / 24:
+// 40.4 / 72.4 and 33.9 / 66.5 us. (With the pairs known but Ls, and with it the pad slice, read at run
+// time, Ls = 16 lost 4% in BF16 at 32^4.)
+#define DWF_PAIR_SPECIALISATIONS(M) M(2) M(3) M(4) M(5) M(6) M(7) M(8) M(9) M(10) M(11) M(12) M(16)
+// Numbers of pairs whose face launches (EPI_HALO, two planes of a block) are specialised too.
+constexpr bool dhop_halo_pairs(int n) { return n == 0 || n == 4 || n == 6 || n == 8; }
+template <int P, int LSHC>
+cudaError_t launch_dhop_pairs(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
+                              cudaStream_t stream);
+#define DWF_DECLARE_PAIRS(N_)                                                                                   \
+  template <>                                                                                                   \
+  cudaError_t launch_dhop_pairs<P32, N_>(const DhopArgs&, bool, bool, int, int, size_t, cudaStream_t);          \
+  template <>                                                                                                   \
+  cudaError_t launch_dhop_pairs<P16, N_>(const DhopArgs&, bool, bool, int, int, size_t, cudaStream_t);          \
+  template <>                                                                                                   \
+  cudaError_t launch_dhop_pairs<PB16, N_>(const DhopArgs&, bool, bool, int, int, size_t, cudaStream_t);
+DWF_DECLARE_PAIRS(0)
+DWF_PAIR_SPECIALISATIONS(DWF_DECLARE_PAIRS)
+#undef DWF_DECLARE_PAIRS
+
 template <int P>
 cudaError_t launch_dhop(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
                         cudaStream_t stream);

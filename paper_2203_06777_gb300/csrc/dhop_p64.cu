@@ -177,48 +177,6 @@ __device__ __forceinline__ long long fx_asr(long long v, int d) {
 // a + v with the sign of v flipped where m is -1 (m is 0 or -1)
 __device__ __forceinline__ long long fx_add_signed(long long a, long long v, long long m) { return a + (v ^ m) + (m & 1); }
 
-// mooee_inv_line for FP64 with one FMA per recurrence step (v inv_d is formed once and used by both
-// sweeps): 3 FP64 instructions per value instead of 4. LS > 0: the line in registers.
-template <int LS>
-__device__ __forceinline__ void mooee_inv_line64(double* v, int Ls_rt, bool forward_form, double mass, double inv_d,
-                                                 double inv_den) {
-  constexpr int S = INV_SLICE_STRIDE;
-  const int Ls = LS > 0 ? LS : Ls_rt;
-  // the mirror form is the forward form on the reversed line
-  double* base = forward_form ? v : v + (Ls - 1) * S;
-  const int st = forward_form ? S : -S;
-  if constexpr (LS > 0) {
-    double w[LS];
-    const double v0 = base[0];
-    double acc = 0;
-#pragma unroll
-    for (int k = 1; k < LS; ++k) {
-      w[k] = base[k * st] * inv_d;
-      acc = fma(acc, inv_d, w[k]);
-    }
-    double y = fma(-mass, acc, v0) * inv_den;
-    base[0] = y;
-#pragma unroll
-    for (int k = 1; k < LS; ++k) {
-      y = fma(y, inv_d, w[k]);
-      base[k * st] = y;
-    }
-  } else {
-    double acc = 0;
-    for (int k = 1; k < Ls; ++k) {
-      const double w = base[k * st] * inv_d;
-      base[k * st] = w;
-      acc = fma(acc, inv_d, w);
-    }
-    double y = fma(-mass, acc, base[0]) * inv_den;
-    base[0] = y;
-    for (int k = 1; k < Ls; ++k) {
-      y = fma(y, inv_d, base[k * st]);
-      base[k * st] = y;
-    }
-  }
-}
-
 // 80 registers: six CTAs of 128 threads per SM. 16^4 x 16 Mpc^+ Mpc at 72 / 80 / 96 / 128 registers:
 // 1001 / 1016 / 1032 / 1070 us, 24^4 x 12: 4200 / 4146 / 4197 / 4330 us; the next hop's loads issued
 // before this hop's products (24 more registers) 1080-1110 us.

@@ -1,12 +1,13 @@
-// Instantiates launch_dhop<DWF_PREC> of a packed precision (FP32, FP16, BF16): one translation
-// unit per precision so that the kernel variants compile in parallel.
+// Instantiates launch_dhop_pairs<DWF_PREC, DWF_PAIRS> of a packed precision (P32, P16, PB16) and
+// extent Ls = 2 DWF_PAIRS (0: any Ls). The build compiles this file once for each of them (both macros are
+// given on the command line), in parallel.
 #include "dhop_kernel.cuh"
 
 namespace gdwf {
 
-template <bool DAG, bool C12, int LSC, int EK>
+template <bool DAG, bool C12, int EK>
 static cudaError_t launch_one(const DhopArgs& a, int threads, int blocks, size_t smem, cudaStream_t stream) {
-  auto kern = dhop_kernel<DWF_PREC, DAG, C12, LSC, EK>;
+  auto kern = dhop_kernel<DWF_PREC, DAG, C12, DWF_PAIRS, EK>;
   if (smem > 48 * 1024) {
     static size_t configured = 0;  // per instantiation
     if (smem > configured) {
@@ -58,56 +59,42 @@ static cudaError_t launch_one(const DhopArgs& a, int threads, int blocks, size_t
   return cudaGetLastError();
 }
 
-template <int LSC>
-static cudaError_t launch_ls(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
-                             cudaStream_t stream) {
-  {
-    // the instantiation with exactly the epilogue parts this launch uses; the CG epilogues exist
-    // for the launches that use them only: Mpc's second launch (pre-operation Mooee, no dag) with
-    // the norm, Mpc^+'s second launch (Mooee^+, dag) with the update, 18-real links
-    if (a.halo_fwd) {  // a face region of a block of a lattice split in t (plain hop)
-      if (a.pre != PRE_NONE || a.post != POST_NONE || a.red || a.in2) return cudaErrorInvalidValue;
-      if (dag) return c12 ? launch_one<true, true, LSC, EPI_HALO>(a, threads, blocks, smem, stream)
-                          : launch_one<true, false, LSC, EPI_HALO>(a, threads, blocks, smem, stream);
-      return c12 ? launch_one<false, true, LSC, EPI_HALO>(a, threads, blocks, smem, stream)
-                 : launch_one<false, false, LSC, EPI_HALO>(a, threads, blocks, smem, stream);
-    }
-    if (a.red && !c12 && a.pre != PRE_NONE && a.post == POST_NONE) {
-      if (a.r && dag) return launch_one<true, false, LSC, EPI_PRE | EPI_AXPY>(a, threads, blocks, smem, stream);
-      if (!a.r && !dag) return launch_one<false, false, LSC, EPI_PRE | EPI_NORM>(a, threads, blocks, smem, stream);
-      return cudaErrorInvalidValue;
-    }
-    if (a.red) return cudaErrorInvalidValue;
-    const int ek = (a.pre != PRE_NONE ? EPI_PRE : 0) | (a.post != POST_NONE ? EPI_POST : 0);
-#define DWF_EK(K)                                                                             \
-  case K:                                                                                     \
-    if (dag) return c12 ? launch_one<true, true, LSC, K>(a, threads, blocks, smem, stream)    \
-                        : launch_one<true, false, LSC, K>(a, threads, blocks, smem, stream);  \
-    return c12 ? launch_one<false, true, LSC, K>(a, threads, blocks, smem, stream)            \
-               : launch_one<false, false, LSC, K>(a, threads, blocks, smem, stream);
-    switch (ek) {
-      DWF_EK(EPI_NONE)
-      DWF_EK(EPI_PRE)
-      DWF_EK(EPI_POST)
-      DWF_EK(EPI_BOTH)
-    }
-#undef DWF_EK
-  }
-  return cudaErrorInvalidValue;
-}
-
 template <>
-cudaError_t launch_dhop<DWF_PREC>(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
-                                  cudaStream_t stream) {
-  switch (a.g.Ls) {
-#define DWF_CASE(L_) \
-  case L_:           \
-    return launch_ls<L_>(a, dag, c12, threads, blocks, smem, stream);
-    DWF_LS_SPECIALISATIONS(DWF_CASE)
-#undef DWF_CASE
-    default:
-      return launch_ls<0>(a, dag, c12, threads, blocks, smem, stream);
+cudaError_t launch_dhop_pairs<DWF_PREC, DWF_PAIRS>(const DhopArgs& a, bool dag, bool c12, int threads, int blocks,
+                                                   size_t smem, cudaStream_t stream) {
+  // the instantiation with exactly the epilogue parts this launch uses; the CG epilogues exist
+  // for the launches that use them only: Mpc's second launch (pre-operation Mooee, no dag) with
+  // the norm, Mpc^+'s second launch (Mooee^+, dag) with the update, 18-real links
+  if (a.halo_fwd) {  // a face region of a block of a lattice split in t (plain hop)
+    if constexpr (dhop_halo_pairs(DWF_PAIRS)) {
+      if (a.pre != PRE_NONE || a.post != POST_NONE || a.red || a.in2) return cudaErrorInvalidValue;
+      if (dag) return c12 ? launch_one<true, true, EPI_HALO>(a, threads, blocks, smem, stream)
+                          : launch_one<true, false, EPI_HALO>(a, threads, blocks, smem, stream);
+      return c12 ? launch_one<false, true, EPI_HALO>(a, threads, blocks, smem, stream)
+                 : launch_one<false, false, EPI_HALO>(a, threads, blocks, smem, stream);
+    }
+    return cudaErrorInvalidValue;
   }
+  if (a.red && !c12 && a.pre != PRE_NONE && a.post == POST_NONE) {
+    if (a.r && dag) return launch_one<true, false, EPI_PRE | EPI_AXPY>(a, threads, blocks, smem, stream);
+    if (!a.r && !dag) return launch_one<false, false, EPI_PRE | EPI_NORM>(a, threads, blocks, smem, stream);
+    return cudaErrorInvalidValue;
+  }
+  if (a.red) return cudaErrorInvalidValue;
+  const int ek = (a.pre != PRE_NONE ? EPI_PRE : 0) | (a.post != POST_NONE ? EPI_POST : 0);
+#define DWF_EK(K)                                                                         \
+  case K:                                                                                 \
+    if (dag) return c12 ? launch_one<true, true, K>(a, threads, blocks, smem, stream)     \
+                        : launch_one<true, false, K>(a, threads, blocks, smem, stream);   \
+    return c12 ? launch_one<false, true, K>(a, threads, blocks, smem, stream)             \
+               : launch_one<false, false, K>(a, threads, blocks, smem, stream);
+  switch (ek) {
+    DWF_EK(EPI_NONE)
+    DWF_EK(EPI_PRE)
+    DWF_EK(EPI_POST)
+  }
+#undef DWF_EK
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace gdwf
