@@ -2,11 +2,15 @@
 // FP64-accumulated reductions and CG vector updates. All are bandwidth-bound passes over the
 // device field layout described in dwf_common.cuh.
 //
-// Elementwise kernels walk a field in units of 16 values: unit (site, g, q) is reals 8g..8g+7 of
-// both slices of pair q of a site block, in the order [real][slice]. Consecutive threads take
-// consecutive pairs, so every precision's 16-byte vectors are read and written contiguously, and
-// fields of different precisions (whose vectors hold 1, 2 or 4 reals of two slices) can be
-// combined in one pass. Pad slices (odd Ls) are zero and stay zero.
+// Elementwise kernels walk a field in units of 16 values: reals 8g..8g+7 of both slices of one pair
+// of a site, in the order [real][slice], NV = 8 / RV vectors. Units are numbered [site block][g 0..2]
+// [site in block][pair q]: with n = 4 Lsh columns, unit u lies in row u / n and column u % n, and its
+// vectors at row * NV chunk strides + column * 16 bytes (+ v chunk strides). Consecutive threads take
+// consecutive columns, so every precision's 16-byte vectors are read and written contiguously, and
+// fields of different precisions (whose vectors hold 1, 2 or 4 reals of two slices) can be combined in
+// one pass. One division by n finds a unit, as a multiplication by 2^64 / n: two 64-bit divisions
+// per unit (~100 instructions each) cost the 16-bit passes most (conversion, norm and inner product of
+// BF16 full fields at 24^4 x 12: 527 -> 489 us). Pad slices (odd Ls) are zero and stay zero.
 #include "dhop_kernel.cuh"
 #include "site_ops.cuh"
 
@@ -15,51 +19,59 @@ namespace gdwf {
 template <int P>
 using RT = typename Store<P>::R;
 
-template <int P>
-__device__ __forceinline__ const char* site_ptr(const void* base, long site, int Lsh) {
-  return static_cast<const char*>(base) + site_offset(site, Lsh, (size_t)Lsh * 2 * 24 * sizeof(typename Store<P>::T));
+// Where a unit lies: row (block and g) and column (site in block and pair) of the unit array.
+struct UnitMap {
+  uint64_t m;      // ceil(2^64 / columns)
+  uint32_t cols;   // 4 Lsh
+  long units;      // 3 nsites Lsh (nsites a multiple of 4)
+};
+
+static inline UnitMap unit_map(long nsites, int Ls) {
+  UnitMap u;
+  u.cols = (uint32_t)(SITE_BLOCK * ls_half(Ls));
+  u.m = ~0ull / u.cols + 1;  // u * cols < 2^64 for every u < 2^56, so that the quotient is exact
+  u.units = nsites * 3 * ls_half(Ls);
+  return u;
 }
 
-// The 16 values of unit (site, g, q): NV = 8 / RV vectors, chunks g*NV .. g*NV + NV - 1.
+// Byte offset of the first of unit u's vectors for a field whose units are NV vectors, and the step
+// between its vectors.
+template <int P>
+__device__ __forceinline__ size_t unit_offset(const UnitMap& um, long u) {
+  constexpr int NV = 16 / Store<P>::VEC;
+  const uint64_t row = __umul64hi((uint64_t)u, um.m);
+  const uint32_t col = (uint32_t)u - (uint32_t)row * um.cols;
+  return ((size_t)row * (NV * um.cols) + col) * 16;
+}
+
+// The 16 values of unit u.
 template <int P, bool COHERENT>
-__device__ __forceinline__ void ld_unit(const void* base, long site, int g, int q, int Lsh, RT<P>* o) {
+__device__ __forceinline__ void ld_unit(const void* base, const UnitMap& um, long u, RT<P>* o) {
   constexpr int VEC = Store<P>::VEC;
-  constexpr int NV = 16 / VEC;
-  const char* sb = site_ptr<P>(base, site, Lsh);
+  const char* p = static_cast<const char*>(base) + unit_offset<P>(um, u);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    const char* p = sb + (g * NV + v) * chunk_stride(Lsh) + (size_t)q * 16;
+  for (int v = 0; v < 16 / VEC; ++v) {
     if (COHERENT)
-      ld16c<P>(p, o + v * VEC);
+      ld16c<P>(p + v * um.cols * 16, o + v * VEC);
     else
-      ld16<P>(p, o + v * VEC);
+      ld16<P>(p + v * um.cols * 16, o + v * VEC);
   }
 }
 
 template <int P>
-__device__ __forceinline__ void st_unit(void* base, long site, int g, int q, int Lsh, const RT<P>* o) {
+__device__ __forceinline__ void st_unit(void* base, const UnitMap& um, long u, const RT<P>* o) {
   constexpr int VEC = Store<P>::VEC;
-  constexpr int NV = 16 / VEC;
-  char* sb = const_cast<char*>(site_ptr<P>(base, site, Lsh));
+  char* p = static_cast<char*>(base) + unit_offset<P>(um, u);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) st16<P>(sb + (g * NV + v) * chunk_stride(Lsh) + (size_t)q * 16, o + v * VEC);
+  for (int v = 0; v < 16 / VEC; ++v) st16<P>(p + v * um.cols * 16, o + v * VEC);
 }
 
 template <int P>
-__device__ __forceinline__ void st_unit_d(void* base, long site, int g, int q, int Lsh, const double* o) {
+__device__ __forceinline__ void st_unit_d(void* base, const UnitMap& um, long u, const double* o) {
   constexpr int VEC = Store<P>::VEC;
-  constexpr int NV = 16 / VEC;
-  char* sb = const_cast<char*>(site_ptr<P>(base, site, Lsh));
+  char* p = static_cast<char*>(base) + unit_offset<P>(um, u);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) st16d<P>(sb + (g * NV + v) * chunk_stride(Lsh) + (size_t)q * 16, o + v * VEC);
-}
-
-// Value i of a unit is real 8g + (i >> 1) of slice 2q + (i & 1).
-__device__ __forceinline__ void unit_coords(long u, int Lsh, long& site, int& g, int& q) {
-  const long rem = u / Lsh;
-  q = (int)(u - rem * Lsh);
-  site = rem / 3;
-  g = (int)(rem - site * 3);
+  for (int v = 0; v < 16 / VEC; ++v) st16d<P>(p + v * um.cols * 16, o + v * VEC);
 }
 
 static inline int grid_for(long n, int threads) {
@@ -271,37 +283,33 @@ cudaError_t launch_pack_gauge(int prec, bool c12, const Geom& g, const double* c
 // ---------------------------------------------------------------- precision conversion
 
 template <int PS, int PD>
-__global__ void k_convert(const void* src, void* dst, long nsites, int Ls, const double* scale_dev, double scale) {
+__global__ void k_convert(const void* src, void* dst, UnitMap um, const double* scale_dev, double scale) {
   using RS = RT<PS>;
   using RD = RT<PD>;
   const double sc = scale_dev ? *scale_dev : scale;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RS a[16];
-    ld_unit<PS, false>(src, site, g, q, Lsh, a);
+    ld_unit<PS, false>(src, um, u, a);
     if constexpr (PS == P64 || PD == P64) {
       double b[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) b[j] = (double)a[j] * sc;
-      st_unit_d<PD>(dst, site, g, q, Lsh, b);
+      st_unit_d<PD>(dst, um, u, b);
     } else {
       RD b[16];
       const float f = (float)sc;
 #pragma unroll
       for (int j = 0; j < 16; ++j) b[j] = (RD)((float)a[j] * f);
-      st_unit<PD>(dst, site, g, q, Lsh, b);
+      st_unit<PD>(dst, um, u, b);
     }
   }
 }
 
 cudaError_t launch_convert(int psrc, int pdst, const void* src, void* dst, long nsites, int Ls, const double* scale_dev,
                            double scale, cudaStream_t st) {
-  const int blocks = grid_for(nsites * 3 * ls_half(Ls), 256);
-#define CV(A, B) k_convert<A, B><<<blocks, 256, 0, st>>>(src, dst, nsites, Ls, scale_dev, scale)
+  const UnitMap um = unit_map(nsites, Ls);
+  const int blocks = grid_for(um.units, 256);
+#define CV(A, B) k_convert<A, B><<<blocks, 256, 0, st>>>(src, dst, um, scale_dev, scale)
 #define CVROW(A)            \
   switch (pdst) {           \
     case P64: CV(A, P64); break;  \
@@ -322,10 +330,151 @@ cudaError_t launch_convert(int psrc, int pdst, const void* src, void* dst, long 
 
 // ---------------------------------------------------------------- standalone Mooee / Mooee^-1
 
-// One CTA holds `spc` whole sites in shared memory (FP32 or FP64 arithmetic): load, apply the
-// fifth-dimension operator, store. in and out may be the same buffer.
+// Up to 32 slice pairs (FP64: the forward operator; the inverse's scan takes 13 FP64 instructions per
+// vector against 6 of the two serial sweeps): one thread per 16-byte vector (both slices of pair q for RV reals of one
+// site), a site's pairs being consecutive lanes of one warp, so that the coupling to slices s -+ 1 and
+// the inverse's recurrence run on shuffles and the field moves through registers once. The inverse
+// of the chirality coupled to s - 1 is, with S_s = sum_{1 <= k <= s} b_k d^-(s-k+1),
+//   y_0 = (b_0 - m S_{Ls-1}) / (d + m d^-(Ls-1)),  y_s = S_s + d^-s y_0,
+// S by a scan over the lanes; y so formed on the pair before feeds the recurrence y_s = (b_s + y_{s-1}) / d
+// over a pair's own slices (its rounding damped by 1 / d). The other chirality is the mirror image in s. Bound by memory in FP32 and 16 bits: inverse at 24^4 x 12 full, FP32, 192 -> 129 us (5.9 TB/s),
+// forward half field 84 -> 59 us. The shared-memory
+// kernel below, which served every case before, stages the field between barriers and runs each
+// line's two sweeps serially. Without the compile-time number of scan steps: 174 us.
+struct InvPowers {
+  double p[65];              // d^-n
+  float inv_lo, inv_den_lo;  // 1 / d and 1 / (d + m d^-(Ls-1)) less their FP32 roundings
+};
+
+// STEPS = ceil(log2 pairs), ODD = odd Ls (slice 2q + 1 of the last pair is the zero pad).
+template <int P, int STEPS, bool ODD>
+__global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, uint32_t groups, int Ls, int gpw, bool dag,
+                                                   bool inverse, double d5, double mass, double inv_den,
+                                                   const __grid_constant__ InvPowers pw) {
+  using R = RT<P>;
+  constexpr int VEC = Store<P>::VEC, RV = Store<P>::RV, NCH = Store<P>::NCH;
+  constexpr int U = P == P64 ? 4 : 2;  // vectors per thread
+  const int Lsh = ls_half(Ls);
+  const int lane = threadIdx.x & 31;
+  const int gl = lane / Lsh, q = lane - gl * Lsh;
+  const uint32_t g0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (uint32_t)(U * gpw) + gl;
+  __shared__ R pws[65];
+  if (threadIdx.x < 65) pws[threadIdx.x] = (R)pw.p[threadIdx.x];
+  R v[U][VEC];
+  bool act[U];
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const uint32_t G = g0 + j * gpw;  // (site block, chunk, site in block)
+    act[j] = gl < gpw && G < groups;
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) v[j][i] = R(0);
+    if (act[j]) ld16c<P>(in + ((size_t)G * Lsh + q) * 16, v[j]);
+  }
+  __syncthreads();
+  const R d = R(d5), m = R(mass);
+  const bool pad_pair = ODD && q == Lsh - 1;
+#pragma unroll
+  for (int j = 0; j < U; ++j) {
+    const uint32_t G = g0 + j * gpw;
+    const bool upper = (G >> 2) % (uint32_t)NCH < NCH / 2;
+    const bool fwd = dag != upper;  // coupled to s - 1
+    if (!inverse) {
+      // o_s = d b_s + c b_{s -+ 1}, c = -1, and m where it wraps around; the lane that holds the
+      // pair before this one in the direction of the coupling, cyclically:
+      const int src = fwd ? (q > 0 ? lane - 1 : lane + Lsh - 1) : (q < Lsh - 1 ? lane + 1 : lane - (Lsh - 1));
+      const R c = (fwd ? q == 0 : q == Lsh - 1) ? m : R(-1);
+#pragma unroll
+      for (int r = 0; r < RV; ++r) {
+        const R a = v[j][2 * r], b = v[j][2 * r + 1];
+        // the slice nearest to the neighbour: the second (first), the only one where the pair ends in the pad
+        const R o = __shfl_sync(0xffffffffu, fwd && !pad_pair ? b : a, src & 31);
+        // one product and two FMAs per vector, whichever way it couples (FP64 fields are bound by that
+        // pipe): the slice coupled to the neighbour's, and the one coupled to it
+        const bool first = fwd || pad_pair;
+        const R p = first ? a : b, n = first ? b : a;
+        const R at_p = d * p + c * o, at_n = d * n - p;
+        const R x = first ? at_p : at_n, y = first ? at_n : at_p;
+        v[j][2 * r] = x;
+        v[j][2 * r + 1] = pad_pair ? R(0) : y;
+      }
+    } else {
+      // position of the pair along the line (0: the one with the slice that the other terms feed into),
+      // and of its first slice in line order (-1: the pad, where the line starts beside it)
+      const int pos = fwd ? q : Lsh - 1 - q;
+      const bool pad_line = ODD && !fwd;
+      const bool head = pos == 0, pad_head = pad_line && head;
+      const int p0 = pad_line ? 2 * pos - 1 : 2 * pos;
+      const int back = fwd ? -1 : 1;
+      const int head_lane = (lane - q + (fwd ? 0 : Lsh - 1)) & 31, tail_lane = (lane - q + (fwd ? Lsh - 1 : 0)) & 31;
+      // 1 / d as an FP32 pair: the two last steps of every slice carry no error of the constant
+      const R inv_d = pws[1], inv_lo = (R)pw.inv_lo;
+      const R cb = pad_head ? R(1) : pws[p0 + 1];
+      R cs[STEPS > 0 ? STEPS : 1];
+#pragma unroll
+      for (int k = 0; k < STEPS; ++k) cs[k] = pos >= (1 << k) ? pws[2 << k] : R(0);
+      const R cp = head ? R(0) : inv_d;
+      const R inv_dn = R(inv_den), inv_dn_lo = (R)pw.inv_den_lo;
+      auto over_den = [&](R t) { return P == P64 ? t * inv_dn : t * inv_dn + t * inv_dn_lo; };
+      auto over_d = [&](R t) { return P == P64 ? t * inv_d : t * inv_d + t * inv_lo; };
+#pragma unroll
+      for (int r = 0; r < RV; ++r) {
+        const R a = fwd ? v[j][2 * r] : v[j][2 * r + 1];  // in line order
+        const R b = fwd ? v[j][2 * r + 1] : v[j][2 * r];
+        const R b0 = __shfl_sync(0xffffffffu, pad_line ? b : a, head_lane);  // the line's first slice
+        // S of the pair's slices: within the pair, then a scan over the pairs before it
+        const R s0l = head ? R(0) : a * inv_d;
+        R s1 = pad_head ? R(0) : (b + s0l) * inv_d;
+#pragma unroll
+        for (int k = 0; k < STEPS; ++k) s1 += cs[k] * __shfl_sync(0xffffffffu, s1, (lane + back * (1 << k)) & 31);
+        // S_{Ls-1}: on the line's last pair, its second slice unless that is the pad
+        R last = s1;
+        if (ODD) {
+          const R s0 = s0l + cp * __shfl_sync(0xffffffffu, s1, (lane + back) & 31);
+          if (fwd) last = s0;
+        }
+        const R y0 = over_den(b0 - m * __shfl_sync(0xffffffffu, last, tail_lane));
+        // y of the pair before, then the recurrence over the pair's own two slices
+        const R prev = __shfl_sync(0xffffffffu, s1 + cb * y0, (lane + back) & 31);
+        const R ya = pad_head ? R(0) : head ? y0 : over_d(a + prev);
+        const R yb = fwd && pad_pair ? R(0) : pad_head ? y0 : over_d(b + ya);
+        v[j][2 * r] = fwd ? ya : yb;
+        v[j][2 * r + 1] = fwd ? yb : ya;
+      }
+    }
+    if (act[j]) st16<P>(out + ((size_t)G * Lsh + q) * 16, v[j]);
+  }
+}
+
 template <int P>
-__global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, long nsites, int Ls, int spc, bool dag,
+static void launch_mooee_vec(const void* in, void* out, long nsites, int Ls, bool dag, bool inverse, double d5,
+                             double mass, double inv_den, const InvPowers& pw, cudaStream_t st) {
+  const int Lsh = ls_half(Ls), gpw = 32 / Lsh;  // lines' vectors per warp
+  const uint32_t groups = (uint32_t)(nsites * Store<P>::NCH);
+  const int blocks = grid_for(groups, 8 * gpw * (P == P64 ? 4 : 2));
+  const char* i = static_cast<const char*>(in);
+  char* o = static_cast<char*>(out);
+  int steps = 0;
+  while ((1 << steps) < Lsh) ++steps;
+#define MV(S_)                                                                                                      \
+  case S_:                                                                                                          \
+    if (Ls & 1)                                                                                                     \
+      k_mooee_vec<P, S_, true><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw); \
+    else                                                                                                            \
+      k_mooee_vec<P, S_, false><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw); \
+    break;
+  switch (steps) { MV(0) MV(1) MV(2) MV(3) MV(4) MV(5) }
+#undef MV
+}
+
+// More than 32 pairs, and the FP64 inverse: one CTA holds `spc` whole sites in shared memory (FP32 or FP64 arithmetic):
+// load, apply the fifth-dimension operator, store. in and out may be the same buffer.
+// Unit number of (site, g, pair q).
+__device__ __forceinline__ long unit_of(long site, int g, int q, int Lsh) {
+  return ((site >> 2) * 3 + g) * (SITE_BLOCK * Lsh) + (site & 3) * Lsh + q;
+}
+
+template <int P>
+__global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, UnitMap um, long nsites, int Ls, int spc, bool dag,
                                                bool inverse, double d5, double mass, double inv_d5, double inv_den) {
   using R = RT<P>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -341,7 +490,7 @@ __global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, long n
     const int sl = rem / 3;
     const int g = rem - sl * 3;
     R v[16];
-    ld_unit<P, true>(in, site0 + sl, g, q, Lsh, v);
+    ld_unit<P, true>(in, um, unit_of(site0 + sl, g, q, Lsh), v);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int s = 2 * q + (i & 1);
@@ -354,7 +503,11 @@ __global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, long n
       const int sl = task / 24;
       const int r = task - sl * 24;
       const bool upper = r < 12;
-      mooee_inv_line<R>(sm + (size_t)sl * Ls * S + r, Ls, dag ? !upper : upper, R(mass), R(inv_d5), R(inv_den));
+      R* line = sm + (size_t)sl * Ls * S + r;
+      if constexpr (P == P64)
+        mooee_inv_line64<0>(line, Ls, dag ? !upper : upper, mass, inv_d5, inv_den);
+      else
+        mooee_inv_line<R>(line, Ls, dag ? !upper : upper, R(mass), R(inv_d5), R(inv_den));
     }
     __syncthreads();
     for (int u = threadIdx.x; u < units; u += blockDim.x) {
@@ -368,7 +521,7 @@ __global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, long n
         const int s = 2 * q + (i & 1);
         o[i] = s < Ls ? sm[((size_t)sl * Ls + s) * S + 8 * g + (i >> 1)] : R(0);
       }
-      st_unit<P>(out, site0 + sl, g, q, Lsh, o);
+      st_unit<P>(out, um, unit_of(site0 + sl, g, q, Lsh), o);
     }
     return;
   }
@@ -394,12 +547,27 @@ __global__ void __launch_bounds__(256) k_mooee(const void* in, void* out, long n
       const bool upper = r < 12;
       o[i] = R(d5) * base[s * S + r] + (upper ? c_up * base[s_up * S + r] : c_lo * base[s_lo * S + r]);
     }
-    st_unit<P>(out, site0 + sl, g, q, Lsh, o);
+    st_unit<P>(out, um, unit_of(site0 + sl, g, q, Lsh), o);
   }
 }
 
 cudaError_t launch_mooee(int prec, const void* in, void* out, long nsites, int Ls, bool dag, bool inverse, double d5,
                          double mass, double inv_d5, double inv_den, cudaStream_t st) {
+  const int Lsh = ls_half(Ls);
+  if (Lsh <= 32 && !(prec == P64 && inverse)) {
+    InvPowers pw;
+    pw.p[0] = 1.0;
+    for (int n = 1; n <= 64; ++n) pw.p[n] = pw.p[n - 1] * inv_d5;
+    pw.inv_lo = (float)(inv_d5 - (double)(float)inv_d5);
+    pw.inv_den_lo = (float)(inv_den - (double)(float)inv_den);
+    switch (prec) {
+      case P64: launch_mooee_vec<P64>(in, out, nsites, Ls, dag, inverse, d5, mass, inv_den, pw, st); break;
+      case P32: launch_mooee_vec<P32>(in, out, nsites, Ls, dag, inverse, d5, mass, inv_den, pw, st); break;
+      case P16: launch_mooee_vec<P16>(in, out, nsites, Ls, dag, inverse, d5, mass, inv_den, pw, st); break;
+      default: launch_mooee_vec<PB16>(in, out, nsites, Ls, dag, inverse, d5, mass, inv_den, pw, st); break;
+    }
+    return cudaGetLastError();
+  }
   const size_t rbytes = prec == P64 ? 8 : 4;
   const size_t site_smem = (size_t)Ls * INV_SLICE_STRIDE * rbytes;
   int spc = (int)((48 * 1024) / site_smem);
@@ -407,7 +575,7 @@ cudaError_t launch_mooee(int prec, const void* in, void* out, long nsites, int L
   if (spc < 1) return cudaErrorInvalidValue;
   const size_t smem = spc * site_smem;
   const int blocks = grid_for(nsites, spc);
-#define MO(P_) k_mooee<P_><<<blocks, 256, smem, st>>>(in, out, nsites, Ls, spc, dag, inverse, d5, mass, inv_d5, inv_den)
+#define MO(P_) k_mooee<P_><<<blocks, 256, smem, st>>>(in, out, unit_map(nsites, Ls), nsites, Ls, spc, dag, inverse, d5, mass, inv_d5, inv_den)
   switch (prec) {
     case P64: MO(P64); break;
     case P32: MO(P32); break;
@@ -423,21 +591,16 @@ cudaError_t launch_mooee(int prec, const void* in, void* out, long nsites, int L
 // Sum over 8 reals of a unit: |a|^2, or the complex a^+ b. Lower precisions form the 8-term
 // partial in FP32 and add it to the FP64 accumulator; FP64 data is accumulated in FP64.
 template <int P, bool INNER>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce(const void* a, const void* b, long nsites, int Ls,
+__global__ void __launch_bounds__(RED_THREADS) k_reduce(const void* a, const void* b, UnitMap um,
                                                         double* partials) {
   using R = RT<P>;
   double acc[2] = {0.0, 0.0};
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     R x[16];
-    ld_unit<P, false>(a, site, g, q, Lsh, x);
+    ld_unit<P, false>(a, um, u, x);
     if (INNER) {
       R y[16];
-      ld_unit<P, false>(b, site, g, q, Lsh, y);
+      ld_unit<P, false>(b, um, u, y);
       R re = 0, im = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -469,9 +632,9 @@ cudaError_t launch_reduce(int prec, const void* a, const void* b, long nsites, i
   const bool inner = b != nullptr;
 #define RD(P_)                                                                              \
   if (inner)                                                                                \
-    k_reduce<P_, true><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, nsites, Ls, partials);     \
+    k_reduce<P_, true><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials);     \
   else                                                                                      \
-    k_reduce<P_, false><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, nsites, Ls, partials);
+    k_reduce<P_, false><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials);
   switch (prec) {
     case P64: RD(P64) break;
     case P32: RD(P32) break;
@@ -487,24 +650,18 @@ cudaError_t launch_reduce(int prec, const void* a, const void* b, long nsites, i
 // ---------------------------------------------------------------- CG updates
 
 template <int PX, int PP>
-__global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const void* p, const void* Ap, long nsites,
-                                                       int Ls, const double* scal, double* partials) {
+__global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const void* p, const void* Ap, UnitMap um, const double* scal, double* partials) {
   using RX = RT<PX>;
   using RP = RT<PP>;
   const RX alpha = (RX)scal[S_ALPHA];
   double acc = 0.0;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX xv[16], rv[16];
     RP pv[16], av[16];
-    ld_unit<PX, true>(x, site, g, q, Lsh, xv);
-    ld_unit<PX, true>(r, site, g, q, Lsh, rv);
-    ld_unit<PP, false>(p, site, g, q, Lsh, pv);
-    ld_unit<PP, false>(Ap, site, g, q, Lsh, av);
+    ld_unit<PX, true>(x, um, u, xv);
+    ld_unit<PX, true>(r, um, u, rv);
+    ld_unit<PP, false>(p, um, u, pv);
+    ld_unit<PP, false>(Ap, um, u, av);
     RX t = 0;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -512,8 +669,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const v
       rv[j] -= alpha * (RX)av[j];
       t += rv[j] * rv[j];
     }
-    st_unit<PX>(x, site, g, q, Lsh, xv);
-    st_unit<PX>(r, site, g, q, Lsh, rv);
+    st_unit<PX>(x, um, u, xv);
+    st_unit<PX>(r, um, u, rv);
     acc += (double)t;
   }
   double v[1] = {acc};
@@ -521,23 +678,18 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const v
 }
 
 template <int PX, int PP>
-__global__ void k_cg_p(const void* r, void* p, long nsites, int Ls, const double* scal) {
+__global__ void k_cg_p(const void* r, void* p, UnitMap um, const double* scal) {
   using RX = RT<PX>;
   using RP = RT<PP>;
   const RX beta = (RX)scal[S_BETA];
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX rv[16];
     RP pv[16];
-    ld_unit<PX, false>(r, site, g, q, Lsh, rv);
-    ld_unit<PP, true>(p, site, g, q, Lsh, pv);
+    ld_unit<PX, false>(r, um, u, rv);
+    ld_unit<PP, true>(p, um, u, pv);
 #pragma unroll
     for (int j = 0; j < 16; ++j) pv[j] = (RP)(rv[j] + beta * (RX)pv[j]);
-    st_unit<PP>(p, site, g, q, Lsh, pv);
+    st_unit<PP>(p, um, u, pv);
   }
 }
 
@@ -547,29 +699,23 @@ __global__ void k_cg_p(const void* r, void* p, long nsites, int Ls, const double
 // iteration (with p^+ Ap) instead of eleven. k_cg_x applies the pending x update alone, before a
 // reliable update folds x into the FP64 solution.
 template <int PX, int PP>
-__global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, long nsites, int Ls, const double* scal,
-                                                      double* partials) {
+__global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, UnitMap um, const double* scal, double* partials) {
   using RX = RT<PX>;
   using RP = RT<PP>;
   const RX alpha = (RX)scal[S_ALPHA];
   double acc = 0.0;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX rv[16];
     RP av[16];
-    ld_unit<PX, true>(r, site, g, q, Lsh, rv);
-    ld_unit<PP, false>(Ap, site, g, q, Lsh, av);
+    ld_unit<PX, true>(r, um, u, rv);
+    ld_unit<PP, false>(Ap, um, u, av);
     RX t = 0;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       rv[j] -= alpha * (RX)av[j];
       t += rv[j] * rv[j];
     }
-    st_unit<PX>(r, site, g, q, Lsh, rv);
+    st_unit<PX>(r, um, u, rv);
     acc += (double)t;
   }
   double v[1] = {acc};
@@ -577,29 +723,24 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, l
 }
 
 template <int PX, int PP, bool UPDATE_P>
-__global__ void k_cg_xp(void* x, const void* r, void* p, long nsites, int Ls, const double* scal) {
+__global__ void k_cg_xp(void* x, const void* r, void* p, UnitMap um, const double* scal) {
   using RX = RT<PX>;
   using RP = RT<PP>;
   const RX alpha = (RX)scal[S_ALPHA];
   const RX beta = (RX)scal[S_BETA];
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX xv[16], rv[16];
     RP pv[16];
-    ld_unit<PX, true>(x, site, g, q, Lsh, xv);
-    ld_unit<PP, UPDATE_P>(p, site, g, q, Lsh, pv);  // coherent when p is rewritten
-    if (UPDATE_P) ld_unit<PX, false>(r, site, g, q, Lsh, rv);
+    ld_unit<PX, true>(x, um, u, xv);
+    ld_unit<PP, UPDATE_P>(p, um, u, pv);  // coherent when p is rewritten
+    if (UPDATE_P) ld_unit<PX, false>(r, um, u, rv);
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       xv[j] += alpha * (RX)pv[j];
       if (UPDATE_P) pv[j] = (RP)(rv[j] + beta * (RX)pv[j]);
     }
-    st_unit<PX>(x, site, g, q, Lsh, xv);
-    if (UPDATE_P) st_unit<PP>(p, site, g, q, Lsh, pv);
+    st_unit<PX>(x, um, u, xv);
+    if (UPDATE_P) st_unit<PP>(p, um, u, pv);
   }
 }
 
@@ -613,7 +754,7 @@ cudaError_t launch_cg_xr(int px, int pp, void* x, void* r, const void* p, const 
                          double* partials, double* scal, cudaStream_t st) {
 #define XR(A, B)                                                                                  \
   if (px == A && pp == B) {                                                                       \
-    k_cg_xr<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, r, p, Ap, nsites, Ls, scal, partials);  \
+    k_cg_xr<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, r, p, Ap, unit_map(nsites, Ls), scal, partials);  \
     cudaError_t e = cudaGetLastError();                                                           \
     if (e != cudaSuccess) return e;                                                               \
     return finalize(partials, 1, scal, FIN_BETA, 0, st);                                          \
@@ -627,7 +768,7 @@ cudaError_t launch_cg_r(int px, int pp, void* r, const void* Ap, long nsites, in
                         cudaStream_t st) {
 #define RU(A, B)                                                                             \
   if (px == A && pp == B) {                                                                  \
-    k_cg_r<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(r, Ap, nsites, Ls, scal, partials);    \
+    k_cg_r<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(r, Ap, unit_map(nsites, Ls), scal, partials);    \
     cudaError_t e = cudaGetLastError();                                                      \
     if (e != cudaSuccess) return e;                                                          \
     return finalize(partials, 1, scal, FIN_BETA, 0, st);                                     \
@@ -639,13 +780,14 @@ cudaError_t launch_cg_r(int px, int pp, void* r, const void* Ap, long nsites, in
 
 cudaError_t launch_cg_xp(int px, int pp, void* x, const void* r, void* p, long nsites, int Ls, const double* scal,
                          bool update_p, cudaStream_t st) {
-  const int blocks = grid_for(nsites * 3 * ls_half(Ls), 256);
+  const UnitMap um = unit_map(nsites, Ls);
+  const int blocks = grid_for(um.units, 256);
 #define XP(A, B)                                                                                        \
   if (px == A && pp == B) {                                                                             \
     if (update_p)                                                                                       \
-      k_cg_xp<A, B, true><<<blocks, 256, 0, st>>>(x, r, p, nsites, Ls, scal);                          \
+      k_cg_xp<A, B, true><<<blocks, 256, 0, st>>>(x, r, p, um, scal);                          \
     else                                                                                                \
-      k_cg_xp<A, B, false><<<blocks, 256, 0, st>>>(x, r, p, nsites, Ls, scal);                         \
+      k_cg_xp<A, B, false><<<blocks, 256, 0, st>>>(x, r, p, um, scal);                         \
     return cudaGetLastError();                                                                          \
   }
   CG_PAIRS(XP)
@@ -655,10 +797,11 @@ cudaError_t launch_cg_xp(int px, int pp, void* x, const void* r, void* p, long n
 
 cudaError_t launch_cg_p(int px, int pp, const void* r, void* p, long nsites, int Ls, const double* scal,
                         cudaStream_t st) {
-  const int blocks = grid_for(nsites * 3 * ls_half(Ls), 256);
+  const UnitMap um = unit_map(nsites, Ls);
+  const int blocks = grid_for(um.units, 256);
 #define PU(A, B)                                                              \
   if (px == A && pp == B) {                                                   \
-    k_cg_p<A, B><<<blocks, 256, 0, st>>>(r, p, nsites, Ls, scal);             \
+    k_cg_p<A, B><<<blocks, 256, 0, st>>>(r, p, um, scal);             \
     return cudaGetLastError();                                                \
   }
   CG_PAIRS(PU)
@@ -666,24 +809,19 @@ cudaError_t launch_cg_p(int px, int pp, const void* r, void* p, long nsites, int
   return cudaErrorInvalidValue;
 }
 
-__global__ void __launch_bounds__(RED_THREADS) k_residual64(const void* b, const void* Ax, void* r, long nsites, int Ls,
+__global__ void __launch_bounds__(RED_THREADS) k_residual64(const void* b, const void* Ax, void* r, UnitMap um,
                                                             double* partials) {
   double acc = 0.0;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     double bv[16], av[16];
-    ld_unit<P64, false>(b, site, g, q, Lsh, bv);
-    ld_unit<P64, false>(Ax, site, g, q, Lsh, av);
+    ld_unit<P64, false>(b, um, u, bv);
+    ld_unit<P64, false>(Ax, um, u, av);
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       bv[j] -= av[j];
       acc += bv[j] * bv[j];
     }
-    st_unit<P64>(r, site, g, q, Lsh, bv);
+    st_unit<P64>(r, um, u, bv);
   }
   double v[1] = {acc};
   block_sum<1>(v, partials, RED_BLOCKS);
@@ -691,71 +829,63 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual64(const void* b, const
 
 cudaError_t launch_residual64(const void* b, const void* Ax, void* r, long nsites, int Ls, double* partials,
                               double* scal, int dst, cudaStream_t st) {
-  k_residual64<<<RED_BLOCKS, RED_THREADS, 0, st>>>(b, Ax, r, nsites, Ls, partials);
+  k_residual64<<<RED_BLOCKS, RED_THREADS, 0, st>>>(b, Ax, r, unit_map(nsites, Ls), partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return finalize(partials, 1, scal, FIN_STORE, dst, st);
 }
 
 template <int PY>
-__global__ void k_accum_zero(void* x, void* y, long nsites, int Ls, const double* c_dev) {
+__global__ void k_accum_zero(void* x, void* y, UnitMap um, const double* c_dev) {
   using RY = RT<PY>;
   const double c = *c_dev;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     double xv[16];
     RY yv[16];
-    ld_unit<P64, true>(x, site, g, q, Lsh, xv);
-    ld_unit<PY, true>(y, site, g, q, Lsh, yv);
+    ld_unit<P64, true>(x, um, u, xv);
+    ld_unit<PY, true>(y, um, u, yv);
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       xv[j] += c * (double)yv[j];
       yv[j] = RY(0);
     }
-    st_unit<P64>(x, site, g, q, Lsh, xv);
-    st_unit<PY>(y, site, g, q, Lsh, yv);
+    st_unit<P64>(x, um, u, xv);
+    st_unit<PY>(y, um, u, yv);
   }
 }
 
 cudaError_t launch_accum_zero(int py, void* x, void* y, long nsites, int Ls, const double* c_dev, cudaStream_t st) {
-  const int blocks = grid_for(nsites * 3 * ls_half(Ls), 256);
+  const UnitMap um = unit_map(nsites, Ls);
+  const int blocks = grid_for(um.units, 256);
   switch (py) {
-    case P64: k_accum_zero<P64><<<blocks, 256, 0, st>>>(x, y, nsites, Ls, c_dev); break;
-    case P32: k_accum_zero<P32><<<blocks, 256, 0, st>>>(x, y, nsites, Ls, c_dev); break;
+    case P64: k_accum_zero<P64><<<blocks, 256, 0, st>>>(x, y, um, c_dev); break;
+    case P32: k_accum_zero<P32><<<blocks, 256, 0, st>>>(x, y, um, c_dev); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
 template <int P>
-__global__ void k_axpby(double a, const void* x, double b, void* y, long nsites, int Ls) {
+__global__ void k_axpby(double a, const void* x, double b, void* y, UnitMap um) {
   using R = RT<P>;
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < units; u += (long)gridDim.x * blockDim.x) {
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     R xv[16], yv[16];
-    ld_unit<P, true>(x, site, g, q, Lsh, xv);
-    ld_unit<P, true>(y, site, g, q, Lsh, yv);
+    ld_unit<P, true>(x, um, u, xv);
+    ld_unit<P, true>(y, um, u, yv);
 #pragma unroll
     for (int j = 0; j < 16; ++j) yv[j] = R(a) * xv[j] + R(b) * yv[j];
-    st_unit<P>(y, site, g, q, Lsh, yv);
+    st_unit<P>(y, um, u, yv);
   }
 }
 
 cudaError_t launch_axpby(int p, double a, const void* x, double b, void* y, long nsites, int Ls, cudaStream_t st) {
-  const int blocks = grid_for(nsites * 3 * ls_half(Ls), 256);
+  const UnitMap um = unit_map(nsites, Ls);
+  const int blocks = grid_for(um.units, 256);
   switch (p) {
-    case P64: k_axpby<P64><<<blocks, 256, 0, st>>>(a, x, b, y, nsites, Ls); break;
-    case P32: k_axpby<P32><<<blocks, 256, 0, st>>>(a, x, b, y, nsites, Ls); break;
-    case P16: k_axpby<P16><<<blocks, 256, 0, st>>>(a, x, b, y, nsites, Ls); break;
-    default: k_axpby<PB16><<<blocks, 256, 0, st>>>(a, x, b, y, nsites, Ls); break;
+    case P64: k_axpby<P64><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
+    case P32: k_axpby<P32><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
+    case P16: k_axpby<P16><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
+    default: k_axpby<PB16><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
   }
   return cudaGetLastError();
 }
@@ -782,25 +912,20 @@ constexpr int NOALLOC_MAX_DEVICES = 64;
 static __device__ __align__(256) double g_noalloc_scratch[2 * NOALLOC_MAX_PARTIALS];
 
 template <int P, bool INNER>
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_chunked(const void* a, const void* b, long nsites, int Ls,
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_chunked(const void* a, const void* b, UnitMap um,
                                                                 double* partials, int nblocks) {
   using R = RT<P>;
   double acc[2] = {0.0, 0.0};
-  const int Lsh = ls_half(Ls);
-  const long units = nsites * 3 * Lsh;
   const long first = (long)blockIdx.x * NOALLOC_UNITS_PER_CTA;
 #pragma unroll
   for (int k = 0; k < NOALLOC_UNITS_PER_THREAD; ++k) {
     const long u = first + threadIdx.x + (long)k * RED_THREADS;
-    if (u >= units) break;
-    long site;
-    int g, q;
-    unit_coords(u, Lsh, site, g, q);
+    if (u >= um.units) break;
     R x[16];
-    ld_unit<P, false>(a, site, g, q, Lsh, x);
+    ld_unit<P, false>(a, um, u, x);
     if (INNER) {
       R y[16];
-      ld_unit<P, false>(b, site, g, q, Lsh, y);
+      ld_unit<P, false>(b, um, u, y);
       R re = 0, im = 0;
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -914,11 +1039,12 @@ extern "C" int grid_dwf_inner_noalloc(int precision, const void* a, const void* 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int nb = nblocks > 0 ? (int)nblocks : 1;
   const bool inner = b != nullptr;
+  const UnitMap um = unit_map(nsites, Ls);
 #define NA(P_)                                                                                         \
   if (inner)                                                                                           \
-    k_reduce_chunked<P_, true><<<nb, RED_THREADS, 0, st>>>(a, b, nsites, Ls, scratch, nb);             \
+    k_reduce_chunked<P_, true><<<nb, RED_THREADS, 0, st>>>(a, b, um, scratch, nb);             \
   else                                                                                                 \
-    k_reduce_chunked<P_, false><<<nb, RED_THREADS, 0, st>>>(a, b, nsites, Ls, scratch, nb);
+    k_reduce_chunked<P_, false><<<nb, RED_THREADS, 0, st>>>(a, b, um, scratch, nb);
   switch (precision) {
     case P64: NA(P64) break;
     case P32: NA(P32) break;
