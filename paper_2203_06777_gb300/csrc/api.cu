@@ -37,10 +37,10 @@ struct grid_dwf {
   void* gauge[4][2] = {{nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}, {nullptr, nullptr}};
   void* gauge_fx[2] = {nullptr, nullptr};  // links as integer blocks (the FP64 hop), per parity
   std::map<int, std::pair<void*, size_t>> ws;  // workspace buffers by id
-  double* partials = nullptr;           // reduction partial sums
+  double* partials = nullptr;           // reduction partial sums, then the count of finished CTAs
   double* scal = nullptr;               // CG scalars (device)
   double* host_scal = nullptr;          // pinned mirror of scal
-  // CG: |r|^2 of each inner iteration copied to a pinned ring with an event, so that the host
+  // CG: |r|^2 of each inner iteration stored in a pinned ring, with an event, so that the host
   // reads an iteration's residual while the next iteration is already queued
   static constexpr int RING = 4;
   double* host_ring = nullptr;
@@ -102,12 +102,16 @@ enum WsId : int {
   WS_PF_A32,
   WS_PF_B32,
   WS_CG_RED,
+  WS_SUM_COUNTS,
 };
 
 // Optional CG epilogue of a packed hop (see dhop_kernel.cuh): per-CTA partial sums
-// into red; with r, the update r -= (*coef) * result instead of a stored result.
+// into red, their total finalised as fin; with r, the update r -= (*coef) * result instead of a stored result.
 struct CgEpilogue {
   double* red = nullptr;
+  int total = 0;       // of them
+  unsigned* count = nullptr;
+  Final fin = {};
   float* r = nullptr;
   const double* coef = nullptr;
 };
@@ -267,6 +271,9 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
   a.plane = h->g.Lxh * h->g.L[1] * h->g.L[2];
   a.region_sites = region.nsites;
   a.red = epi.red;
+  a.red_total = epi.total;
+  a.red_count = epi.count;
+  a.fin = epi.fin;
   a.r = epi.r;
   a.axpy_coef = epi.coef;
   a.red_base = 0;
@@ -393,6 +400,26 @@ int mdagm_impl(grid_dwf_t* h, int prec, const void* in, void* out, void* to, voi
   return GRID_DWF_OK;
 }
 
+// A total to scal[dst] (or finalised as kind), and to pinned host memory if host is given.
+Final final_to(const grid_dwf_t* h, int kind, int dst, double* host = nullptr) {
+  return Final{reinterpret_cast<unsigned*>(h->partials + 2 * RED_BLOCKS), h->scal, kind, dst, host};
+}
+
+// Workspaces of finish_grouped_sums for n partial sums: the sums, and the groups' counts (for any n of
+// this lattice; cleared once, every launch leaves them 0).
+int sums_workspace(grid_dwf_t* h, int n, CgEpilogue& epi) {
+  void* p = nullptr;
+  RET(ws_get(h, WS_CG_RED, sizeof(double) * (size_t)(n + sum_groups(n)), &p));
+  epi.red = static_cast<double*>(p);
+  epi.total = n;
+  const bool fresh = h->ws.find(WS_SUM_COUNTS) == h->ws.end();
+  const size_t bytes = sizeof(unsigned) * (size_t)sum_groups(2 * h->g.N4h);
+  RET(ws_get(h, WS_SUM_COUNTS, bytes, &p));
+  epi.count = static_cast<unsigned*>(p);
+  if (fresh) CK(cudaMemsetAsync(p, 0, bytes, h->stream), "partial sums");
+  return GRID_DWF_OK;
+}
+
 int read_scalars(grid_dwf_t* h) {
   CK(cudaMemcpyAsync(h->host_scal, h->scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, h->stream), "scalar read");
   CK(cudaStreamSynchronize(h->stream), "scalar read");
@@ -495,7 +522,8 @@ int grid_dwf_create(const int dims[4], int Ls, double M5, double mass, const int
     int l2 = 0;
     if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, h->device) == cudaSuccess && l2 > 0) h->l2_bytes = (size_t)l2;
   }
-  cudaError_t e = cudaMalloc(&h->partials, sizeof(double) * 2 * RED_BLOCKS);
+  cudaError_t e = cudaMalloc(&h->partials, sizeof(double) * (2 * RED_BLOCKS + 1));
+  if (e == cudaSuccess) e = cudaMemset(h->partials, 0, sizeof(double) * (2 * RED_BLOCKS + 1));
   if (e == cudaSuccess) e = cudaMalloc(&h->scal, sizeof(double) * S_COUNT);
   if (e == cudaSuccess) e = cudaMallocHost(&h->host_scal, sizeof(double) * (2 * S_COUNT + 1));
   if (e == cudaSuccess) e = cudaMallocHost(&h->host_ring, sizeof(double) * grid_dwf::RING);
@@ -696,9 +724,9 @@ int grid_dwf_norm2(grid_dwf_t* h, int precision, int subset, const void* a, doub
     return fail(h, GRID_DWF_ERR_INVALID_ARG, "bad precision/subset/result");
   RET(check_ptr(h, a, "a"));
   const long nsites = (long)h->g.N4h * (subset == GRID_DWF_FULL ? 2 : 1);
-  CK(launch_reduce(precision, a, nullptr, nsites, h->Ls, h->partials, h->scal, FIN_STORE, S_TMP0, h->stream), "norm2");
-  RET(read_scalars(h));
-  *result = h->host_scal[S_TMP0];
+  CK(launch_reduce(precision, a, nullptr, nsites, h->Ls, h->partials, final_to(h, FIN_STORE, S_TMP0, h->host_scal), h->stream), "norm2");
+  CK(cudaStreamSynchronize(h->stream), "norm2");
+  *result = h->host_scal[0];
   return GRID_DWF_OK;
 }
 
@@ -710,10 +738,10 @@ int grid_dwf_inner(grid_dwf_t* h, int precision, int subset, const void* a, cons
   RET(check_ptr(h, a, "a"));
   RET(check_ptr(h, b, "b"));
   const long nsites = (long)h->g.N4h * (subset == GRID_DWF_FULL ? 2 : 1);
-  CK(launch_reduce(precision, a, b, nsites, h->Ls, h->partials, h->scal, FIN_STORE, S_TMP0, h->stream), "inner");
-  RET(read_scalars(h));
-  result[0] = h->host_scal[S_TMP0];
-  result[1] = h->host_scal[S_TMP1];
+  CK(launch_reduce(precision, a, b, nsites, h->Ls, h->partials, final_to(h, FIN_STORE, S_TMP0, h->host_scal), h->stream), "inner");
+  CK(cudaStreamSynchronize(h->stream), "inner");
+  result[0] = h->host_scal[0];
+  result[1] = h->host_scal[1];
   return GRID_DWF_OK;
 }
 
@@ -845,8 +873,8 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
   RET(ws_get(h, WS_CG_AP, hb, &Ap));
   RET(ws_get(h, WS_CG_TO, hb, &to));
   const int P = GRID_DWF_FP64;
-  CK(launch_reduce(P, rhs, nullptr, N, Ls, h->partials, h->scal, FIN_STORE, S_TMP1, h->stream), "cg norm");
-  CK(launch_reduce(P, xo, nullptr, N, Ls, h->partials, h->scal, FIN_STORE, S_TMP0, h->stream), "cg guess norm");
+  CK(launch_reduce(P, rhs, nullptr, N, Ls, h->partials, final_to(h, FIN_STORE, S_TMP1), h->stream), "cg norm");
+  CK(launch_reduce(P, xo, nullptr, N, Ls, h->partials, final_to(h, FIN_STORE, S_TMP0), h->stream), "cg guess norm");
   RET(read_scalars(h));
   const double rhs_norm = std::sqrt(h->host_scal[S_TMP1]);
   double rr;
@@ -859,7 +887,7 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
     // true residual r = rhs - A x_o
     RET(mdagm_impl(h, P, xo, Ap, to, te));
     flops += 4 * half_flops;
-    CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, h->scal, S_RR, h->stream), "cg residual");
+    CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, final_to(h, FIN_STORE, S_RR), h->stream), "cg residual");
     RET(read_scalars(h));
     rr = h->host_scal[S_RR];
   }
@@ -876,8 +904,8 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
     RET(write_scalar(h, S_PSCALE, 1.0));
     while (!converged && iters < maxiter) {
       RET(mdagm_impl(h, P, p, Ap, to, te));
-      CK(launch_reduce(P, p, Ap, N, Ls, h->partials, h->scal, FIN_ALPHA, 0, h->stream), "cg pAp");
-      CK(launch_cg_xr(P, P, xo, r, p, Ap, N, Ls, h->partials, h->scal, h->stream), "cg update");
+      CK(launch_reduce(P, p, Ap, N, Ls, h->partials, final_to(h, FIN_ALPHA, 0), h->stream), "cg pAp");
+      CK(launch_cg_xr(P, P, xo, r, p, Ap, N, Ls, h->partials, final_to(h, FIN_BETA, 0), h->stream), "cg update");
       CK(launch_cg_p(P, P, r, p, N, Ls, h->scal, h->stream), "cg p");
       flops += 4 * half_flops;
       ++iters;
@@ -912,7 +940,7 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
     CK(launch_convert(P, GRID_DWF_FP32, r, rs, N, Ls, nullptr, sigma, h->stream), "cg init");
     CK(launch_convert(GRID_DWF_FP32, PS, rs, ps, N, Ls, nullptr, 1.0, h->stream), "cg init");
     CK(cudaMemsetAsync(xs, 0, hs32, h->stream), "cg init");
-    CK(launch_reduce(GRID_DWF_FP32, rs, nullptr, N, Ls, h->partials, h->scal, FIN_STORE, S_RR, h->stream), "cg init");
+    CK(launch_reduce(GRID_DWF_FP32, rs, nullptr, N, Ls, h->partials, final_to(h, FIN_STORE, S_RR), h->stream), "cg init");
     RET(write_scalar(h, S_PSCALE, 1.0));
     RET(read_scalars(h));
     double rr_s = h->host_scal[S_RR];
@@ -922,14 +950,15 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
     // epilogue of Mpc^+'s second launch, so A p is never stored. Partial sums: one per CTA.
     // Both use the FP32 results before they are rounded to the storage format.
     const bool fused = !h->c12;
-    double* red = nullptr;
-    int nred = 0;
+    CgEpilogue norm, axpy;
     if (fused) {
       const int spc = hop_sites_per_cta(h, PS);
-      nred = (int)(N / spc) + (N % spc ? 1 : 0);  // the full CTAs, and the end CTA if there is one
-      void* rp = nullptr;
-      RET(ws_get(h, WS_CG_RED, sizeof(double) * (size_t)nred, &rp));
-      red = static_cast<double*>(rp);
+      // the full CTAs, and the end CTA if there is one
+      RET(sums_workspace(h, (int)(N / spc) + (N % spc ? 1 : 0), norm));
+      norm.fin = final_to(h, FIN_ALPHA, 0);
+      axpy = norm;
+      axpy.r = static_cast<float*>(rs);
+      axpy.coef = h->scal + S_ALPHA;
     }
     int last_update = 0;  // iteration of the last reliable update (its |r|^2 is on another scale)
     // The decision reads the previous iteration's residual (the GPU never waits for the host)
@@ -938,35 +967,27 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
     // 170 / 169 at the same time; FP16: 171 / 169, and 0.230 s against 0.244 s).
     const int lag = h->cg_lag >= 0 ? h->cg_lag : (PS == GRID_DWF_BF16 ? 0 : 1);
     while (!converged && iters < maxiter) {
+      // |r|^2 of this iteration goes to the host ring as well; the decision below reads the previous
+      // iteration's, which is complete or nearly so while this one is still queued
+      const int slot = (iters + 1) % grid_dwf::RING;
+      const Final beta = final_to(h, FIN_BETA, 0, h->host_ring + slot);
       if (fused) {
-        CgEpilogue norm;
-        norm.red = red;
-        CgEpilogue axpy;
-        axpy.red = red;
-        axpy.r = static_cast<float*>(rs);
-        axpy.coef = h->scal + S_ALPHA;
+        axpy.fin = beta;
         RET(dhop_half(h, PS, ps, tes, 0, false, PRE_NONE, POST_INV, 1.0, 0.0, nullptr));
         RET(dhop_half(h, PS, tes, tos, 1, false, PRE_MOOEE, POST_NONE, -0.25, 1.0, ps, nullptr, nullptr, nullptr, norm));
-        CK(launch_finalize_n(red, nred, h->scal, FIN_ALPHA, 0, h->stream), "cg pAp");
         RET(dhop_half(h, PS, tos, tes, 0, true, PRE_NONE, POST_INV_DAG, 1.0, 0.0, nullptr));
         RET(dhop_half(h, PS, tes, aps, 1, true, PRE_MOOEE_DAG, POST_NONE, -0.25, 1.0, tos, nullptr, nullptr, nullptr,
                       axpy));
-        CK(launch_finalize_n(red, nred, h->scal, FIN_BETA, 0, h->stream), "cg update");
       } else {
         RET(mdagm_impl(h, PS, ps, aps, tos, tes));
-        CK(launch_reduce(PS, ps, aps, N, Ls, h->partials, h->scal, FIN_ALPHA, 0, h->stream), "cg pAp");
+        CK(launch_reduce(PS, ps, aps, N, Ls, h->partials, final_to(h, FIN_ALPHA, 0), h->stream), "cg pAp");
         // r -= alpha Ap now; x += alpha p is deferred to the pass that updates p (one read of p)
-        CK(launch_cg_r(GRID_DWF_FP32, PS, rs, aps, N, Ls, h->partials, h->scal, h->stream), "cg update");
+        CK(launch_cg_r(GRID_DWF_FP32, PS, rs, aps, N, Ls, h->partials, beta, h->stream), "cg update");
       }
       flops += 4 * half_flops;
       ++iters;
       rr_is_true = false;  // x_s has moved since the last true residual
-      // |r|^2 of this iteration to the host ring; the decision below reads the previous
-      // iteration's, which is complete or nearly so while this one is still queued
-      const int slot = iters % grid_dwf::RING;
-      CK(cudaMemcpyAsync(h->host_ring + slot, h->scal + S_RRNEW, sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-         "cg residual copy");
-      CK(cudaEventRecord(h->ring_ev[slot], h->stream), "cg residual copy");
+      CK(cudaEventRecord(h->ring_ev[slot], h->stream), "cg residual");
       bool reliable = iters == maxiter;
       if (iters - lag > last_update) {
         const int prev = (iters - lag) % grid_dwf::RING;
@@ -987,7 +1008,7 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
         CK(launch_accum_zero(GRID_DWF_FP32, xo, xs, N, Ls, h->scal + S_TMP0, h->stream), "cg reliable");
         RET(mdagm_impl(h, P, xo, Ap, to, te));
         flops += 4 * half_flops;
-        CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, h->scal, S_TMP1, h->stream), "cg reliable");
+        CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, final_to(h, FIN_STORE, S_TMP1), h->stream), "cg reliable");
         RET(read_scalars(h));
         ++updates;
         last_update = iters;
@@ -1001,7 +1022,7 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
         }
         const double sigma_new = std::sqrt(nreal) / std::sqrt(rr64);
         CK(launch_convert(P, GRID_DWF_FP32, r, rs, N, Ls, nullptr, sigma_new, h->stream), "cg reliable");
-        CK(launch_reduce(GRID_DWF_FP32, rs, nullptr, N, Ls, h->partials, h->scal, FIN_STORE, S_RR, h->stream),
+        CK(launch_reduce(GRID_DWF_FP32, rs, nullptr, N, Ls, h->partials, final_to(h, FIN_STORE, S_RR), h->stream),
            "cg reliable");
         // beta (true units) = |r_true|^2 / |r_old|^2 with |r_old|^2 = rr_old_s / sigma^2; the stored
         // p carries scale sigma and must move to sigma_new.
@@ -1025,7 +1046,7 @@ int cg_normal(grid_dwf_t* h, const void* rhs, void* xo_, double tol, int maxiter
   if (!rr_is_true) {
     RET(mdagm_impl(h, P, xo, Ap, to, te));
     flops += 4 * half_flops;
-    CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, h->scal, S_TMP0, h->stream), "cg final");
+    CK(launch_residual64(rhs, Ap, r, N, Ls, h->partials, final_to(h, FIN_STORE, S_TMP0), h->stream), "cg final");
     RET(read_scalars(h));
     rr_final = h->host_scal[S_TMP0];
   }
@@ -1103,17 +1124,15 @@ int grid_dwf_force(grid_dwf_t* h, int precision, const void* psi, void* chi, dou
   if (G && (overlap(G, gb, psi, fb) || overlap(G, gb, c, fb))) return fail(h, GRID_DWF_ERR_ALIAS, "force: G overlaps");
   if (precision == GRID_DWF_FP32 && !h->c12) {
     // chi = M psi with |chi|^2 summed in the same launch (one partial per CTA, FP64 across CTAs)
-    const int nred = full_partials(h, precision);
-    void* rp = nullptr;
-    RET(ws_get(h, WS_CG_RED, sizeof(double) * (size_t)nred, &rp));
     CgEpilogue norm;
-    norm.red = static_cast<double*>(rp);
+    RET(sums_workspace(h, full_partials(h, precision), norm));
+    norm.fin = final_to(h, FIN_STORE, S_TMP0, h->host_scal);
     const char* ic = static_cast<const char*>(psi);
     RET(dhop_full(h, precision, ic, static_cast<char*>(c), false, PRE_MOOEE, -0.5, 1.0, ic, norm));
-    CK(launch_finalize_n(norm.red, nred, h->scal, FIN_STORE, S_TMP0, h->stream), "force action");
   } else {
     RET(grid_dwf_m(h, precision, psi, c, 0));
-    CK(launch_reduce(precision, c, nullptr, 2L * h->g.N4h, h->Ls, h->partials, h->scal, FIN_STORE, S_TMP0, h->stream),
+    CK(launch_reduce(precision, c, nullptr, 2L * h->g.N4h, h->Ls, h->partials,
+                     final_to(h, FIN_STORE, S_TMP0, h->host_scal), h->stream),
        "force action");
   }
   RET(ensure_gauge(h, precision));
@@ -1121,8 +1140,8 @@ int grid_dwf_force(grid_dwf_t* h, int precision, const void* psi, void* chi, dou
     CK(launch_force(precision, h->c12, h->g, psi, c, h->gauge[precision][0], h->gauge[precision][1], F, G, 1.0, h->fp64_arith == GRID_DWF_FP64_ARITH_FLOAT_FLOAT,
                     h->stream),
        "force");
-  RET(read_scalars(h));
-  if (S_out) *S_out = h->host_scal[S_TMP0];
+  CK(cudaStreamSynchronize(h->stream), "force");
+  if (S_out) *S_out = h->host_scal[0];
   return finish(h, "force");
 }
 
@@ -1161,7 +1180,7 @@ int grid_dwf_pf_force(grid_dwf_t* h, const void* phi, void* X, double tol, int m
   RET(dhop_half(h, P, Be + hb, Be, 0, true, PRE_NONE, POST_INV_DAG, 1.0, 0.0, nullptr));
   CK(cudaMemcpyAsync(Ae + hb, X, hb, cudaMemcpyDeviceToDevice, h->stream), "pf_force copy");
   // S = Re phi^+ X (phi^+ X is real for the Hermitian positive Mpc^+ Mpc)
-  CK(launch_reduce(P, phi, X, N, Ls, h->partials, h->scal, FIN_STORE, S_TMP0, h->stream), "pf_force action");
+  CK(launch_reduce(P, phi, X, N, Ls, h->partials, final_to(h, FIN_STORE, S_TMP0), h->stream), "pf_force action");
   if (F || G) {
     const void* a = A;
     const void* b = B;

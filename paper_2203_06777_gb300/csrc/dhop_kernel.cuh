@@ -29,6 +29,7 @@
 #pragma once
 
 #include "dwf_common.cuh"
+#include "site_ops.cuh"
 
 namespace gdwf {
 
@@ -72,6 +73,9 @@ struct DhopArgs {
   int region_sites;
   double* red;
   int red_base;
+  unsigned* red_count;
+  int red_total;       // partial sums of the launches together; the last one finalises their total as fin
+  Final fin;
   int own_from;
   float* r;            // EPI_AXPY: FP32 half field updated in place, r -= (*axpy_coef) * (hopping result)
   const double* axpy_coef;
@@ -748,22 +752,6 @@ __device__ __forceinline__ void mooee_inv_line_vec(float* line, bool forward_for
 //                 planes only (the interior needs no halo and runs the plain instantiation).
 enum EpiKind : int { EPI_NONE = 0, EPI_PRE = 1, EPI_POST = 2, EPI_BOTH = 3, EPI_NORM = 4, EPI_AXPY = 8, EPI_HALO = 16 };
 
-// Sum of one value per thread over the CTA in a fixed order (warp shuffles, then the warps in
-// order), written by thread 0 to *dst.
-__device__ __forceinline__ void cta_sum_to(double v, double* dst) {
-  __shared__ double wsum[32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) wsum[warp] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += wsum[w];
-    *dst = t;
-  }
-}
-
 // FP32 / FP16 / BF16: one thread per (site, slice pair), packed two-wide arithmetic.
 template <int P, bool DAG, bool C12, int LSHC, int EK>
 __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
@@ -972,7 +960,8 @@ __device__ __forceinline__ void dhop_body_pair(const DhopArgs& a) {
 #pragma unroll
         for (int r = 0; r < 24; ++r) n2 = fmaf(acc[r].x, acc[r].x, fmaf(acc[r].y, acc[r].y, n2));
       }
-      cta_sum_to(owned ? (double)n2 : 0.0, a.red + a.red_base + (int)blockIdx.x);
+      const double sum = cta_sum(owned ? (double)n2 : 0.0);
+      finish_grouped_sums(a.red, a.red_count, a.red_total, a.red_base + (int)blockIdx.x, sum, a.fin);
     } else {
       store_pair<P, LSHC>(outb, q, Lsh, acc);
     }

@@ -104,78 +104,6 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* partials, int 
   }
 }
 
-// Second pass: one CTA sums the RED_BLOCKS partials in a fixed order.
-__global__ void __launch_bounds__(RED_THREADS) k_finalize(const double* partials, int ncomp, double* scal, int kind,
-                                                         int dst) {
-  __shared__ double red[2][RED_THREADS];
-  for (int k = 0; k < ncomp; ++k) {
-    double t = 0;
-    for (int i = threadIdx.x; i < RED_BLOCKS; i += RED_THREADS) t += partials[k * RED_BLOCKS + i];
-    red[k][threadIdx.x] = t;
-  }
-  __syncthreads();
-  for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w)
-      for (int k = 0; k < ncomp; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double tot = red[0][0];
-    if (kind == FIN_STORE) {
-      scal[dst] = tot;
-      if (ncomp > 1) scal[dst + 1] = red[1][0];
-    } else if (kind == FIN_ALPHA) {
-      scal[S_PAP] = tot;
-      scal[S_ALPHA] = scal[S_RR] / tot;
-    } else if (kind == FIN_BETA) {
-      scal[S_RRNEW] = tot;
-      scal[S_BETA] = scal[S_PSCALE] * tot / scal[S_RR];
-      scal[S_RROLD] = scal[S_RR];
-      scal[S_RR] = tot;
-      scal[S_PSCALE] = 1.0;
-    }
-  }
-}
-
-static cudaError_t finalize(const double* partials, int ncomp, double* scal, int kind, int dst, cudaStream_t st) {
-  k_finalize<<<1, RED_THREADS, 0, st>>>(partials, ncomp, scal, kind, dst);
-  return cudaGetLastError();
-}
-
-// n partials (any n) summed in a fixed order: thread t takes t, t + RED_THREADS, ..., then a tree.
-__global__ void __launch_bounds__(RED_THREADS) k_finalize_n(const double* partials, int n, double* scal, int kind,
-                                                           int dst) {
-  __shared__ double red[RED_THREADS];
-  double t = 0;
-  for (int i = threadIdx.x; i < n; i += RED_THREADS) t += partials[i];
-  red[threadIdx.x] = t;
-  __syncthreads();
-  for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double tot = red[0];
-    if (kind == FIN_STORE) {
-      scal[dst] = tot;
-    } else if (kind == FIN_ALPHA) {
-      scal[S_PAP] = tot;
-      scal[S_ALPHA] = scal[S_RR] / tot;
-    } else if (kind == FIN_BETA) {
-      scal[S_RRNEW] = tot;
-      scal[S_BETA] = scal[S_PSCALE] * tot / scal[S_RR];
-      scal[S_RROLD] = scal[S_RR];
-      scal[S_RR] = tot;
-      scal[S_PSCALE] = 1.0;
-    }
-  }
-}
-
-cudaError_t launch_finalize_n(const double* partials, int n, double* scal, int kind, int dst, cudaStream_t st) {
-  k_finalize_n<<<1, RED_THREADS, 0, st>>>(partials, n, scal, kind, dst);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- pack / unpack
 
 template <int P>
@@ -679,7 +607,7 @@ cudaError_t launch_mooee(int prec, const void* in, void* out, long nsites, int L
 // partial in FP32 and add it to the FP64 accumulator; FP64 data is accumulated in FP64.
 template <int P, bool INNER>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce(const void* a, const void* b, UnitMap um,
-                                                        double* partials) {
+                                                        double* partials, const Final f) {
   using R = RT<P>;
   double acc[2] = {0.0, 0.0};
   for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
@@ -708,20 +636,22 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce(const void* a, const voi
   }
   if (INNER) {
     block_sum<2>(acc, partials, RED_BLOCKS);
+    finish_sums<2>(partials, RED_BLOCKS, f);
   } else {
     double v[1] = {acc[0]};
     block_sum<1>(v, partials, RED_BLOCKS);
+    finish_sums<1>(partials, RED_BLOCKS, f);
   }
 }
 
-cudaError_t launch_reduce(int prec, const void* a, const void* b, long nsites, int Ls, double* partials, double* scal,
-                          int kind, int dst, cudaStream_t st) {
+cudaError_t launch_reduce(int prec, const void* a, const void* b, long nsites, int Ls, double* partials, const Final& f,
+                          cudaStream_t st) {
   const bool inner = b != nullptr;
 #define RD(P_)                                                                              \
   if (inner)                                                                                \
-    k_reduce<P_, true><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials);     \
+    k_reduce<P_, true><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials, f);     \
   else                                                                                      \
-    k_reduce<P_, false><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials);
+    k_reduce<P_, false><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, unit_map(nsites, Ls), partials, f);
   switch (prec) {
     case P64: RD(P64) break;
     case P32: RD(P32) break;
@@ -729,18 +659,16 @@ cudaError_t launch_reduce(int prec, const void* a, const void* b, long nsites, i
     default: RD(PB16) break;
   }
 #undef RD
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return finalize(partials, inner ? 2 : 1, scal, kind, dst, st);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- CG updates
 
 template <int PX, int PP>
-__global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const void* p, const void* Ap, UnitMap um, const double* scal, double* partials) {
+__global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const void* p, const void* Ap, UnitMap um, double* partials, const Final f) {
   using RX = RT<PX>;
   using RP = RT<PP>;
-  const RX alpha = (RX)scal[S_ALPHA];
+  const RX alpha = (RX)f.scal[S_ALPHA];
   double acc = 0.0;
   for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX xv[16], rv[16];
@@ -762,6 +690,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_xr(void* x, void* r, const v
   }
   double v[1] = {acc};
   block_sum<1>(v, partials, RED_BLOCKS);
+  finish_sums<1>(partials, RED_BLOCKS, f);
 }
 
 template <int PX, int PP>
@@ -786,10 +715,10 @@ __global__ void k_cg_p(const void* r, void* p, UnitMap um, const double* scal) {
 // iteration (with p^+ Ap) instead of eleven. k_cg_x applies the pending x update alone, before a
 // reliable update folds x into the FP64 solution.
 template <int PX, int PP>
-__global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, UnitMap um, const double* scal, double* partials) {
+__global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, UnitMap um, double* partials, const Final f) {
   using RX = RT<PX>;
   using RP = RT<PP>;
-  const RX alpha = (RX)scal[S_ALPHA];
+  const RX alpha = (RX)f.scal[S_ALPHA];
   double acc = 0.0;
   for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     RX rv[16];
@@ -807,6 +736,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_r(void* r, const void* Ap, U
   }
   double v[1] = {acc};
   block_sum<1>(v, partials, RED_BLOCKS);
+  finish_sums<1>(partials, RED_BLOCKS, f);
 }
 
 template <int PX, int PP, bool UPDATE_P>
@@ -838,27 +768,23 @@ __global__ void k_cg_xp(void* x, const void* r, void* p, UnitMap um, const doubl
   M(P32, PB16)
 
 cudaError_t launch_cg_xr(int px, int pp, void* x, void* r, const void* p, const void* Ap, long nsites, int Ls,
-                         double* partials, double* scal, cudaStream_t st) {
+                         double* partials, const Final& f, cudaStream_t st) {
 #define XR(A, B)                                                                                  \
   if (px == A && pp == B) {                                                                       \
-    k_cg_xr<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, r, p, Ap, unit_map(nsites, Ls), scal, partials);  \
-    cudaError_t e = cudaGetLastError();                                                           \
-    if (e != cudaSuccess) return e;                                                               \
-    return finalize(partials, 1, scal, FIN_BETA, 0, st);                                          \
+    k_cg_xr<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(x, r, p, Ap, unit_map(nsites, Ls), partials, f);  \
+    return cudaGetLastError();                                                                    \
   }
   CG_PAIRS(XR)
 #undef XR
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_cg_r(int px, int pp, void* r, const void* Ap, long nsites, int Ls, double* partials, double* scal,
+cudaError_t launch_cg_r(int px, int pp, void* r, const void* Ap, long nsites, int Ls, double* partials, const Final& f,
                         cudaStream_t st) {
 #define RU(A, B)                                                                             \
   if (px == A && pp == B) {                                                                  \
-    k_cg_r<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(r, Ap, unit_map(nsites, Ls), scal, partials);    \
-    cudaError_t e = cudaGetLastError();                                                      \
-    if (e != cudaSuccess) return e;                                                          \
-    return finalize(partials, 1, scal, FIN_BETA, 0, st);                                     \
+    k_cg_r<A, B><<<RED_BLOCKS, RED_THREADS, 0, st>>>(r, Ap, unit_map(nsites, Ls), partials, f);    \
+    return cudaGetLastError();                                                               \
   }
   CG_PAIRS(RU)
 #undef RU
@@ -897,7 +823,7 @@ cudaError_t launch_cg_p(int px, int pp, const void* r, void* p, long nsites, int
 }
 
 __global__ void __launch_bounds__(RED_THREADS) k_residual64(const void* b, const void* Ax, void* r, UnitMap um,
-                                                            double* partials) {
+                                                            double* partials, const Final f) {
   double acc = 0.0;
   for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
     double bv[16], av[16];
@@ -912,14 +838,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual64(const void* b, const
   }
   double v[1] = {acc};
   block_sum<1>(v, partials, RED_BLOCKS);
+  finish_sums<1>(partials, RED_BLOCKS, f);
 }
 
 cudaError_t launch_residual64(const void* b, const void* Ax, void* r, long nsites, int Ls, double* partials,
-                              double* scal, int dst, cudaStream_t st) {
-  k_residual64<<<RED_BLOCKS, RED_THREADS, 0, st>>>(b, Ax, r, unit_map(nsites, Ls), partials);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return finalize(partials, 1, scal, FIN_STORE, dst, st);
+                              const Final& f, cudaStream_t st) {
+  k_residual64<<<RED_BLOCKS, RED_THREADS, 0, st>>>(b, Ax, r, unit_map(nsites, Ls), partials, f);
+  return cudaGetLastError();
 }
 
 template <int PY>
