@@ -13,8 +13,8 @@
 // Because (1 -+ gamma_mu)/2 is a rank-2 projector, each spin sum is the sum over the two spins
 // of the projected half spinors: sum_spin a (x) [(1 - gamma) b]^+ = sum_{h=0,1} (P a)_h (x) (P b)_h^*.
 //
-// Thread mapping, as in the hopping kernel: one thread per (4D site, slice pair) for FP32 fields
-// and per (4D site, slice) for FP64, whole sites per CTA, one parity per grid row. For each mu the
+// Thread mapping, as in the hopping kernels: one thread per (4D site, slice pair) for FP32 fields
+// and two per (4D site, slice) for FP64, whole sites per CTA, one parity per grid row. For each mu the
 // threads form their slices' contributions to B1 and B2 of the link U_mu(x) leaving their site
 // (the own spinors and the two x + mu neighbours, the same loads as one Dhop hop), the CTA sums
 // them over the site's slices through shared memory, and the link algebra is spread over the
@@ -22,17 +22,17 @@
 // at most 8 slice pairs and the block sums in FP64, and the link algebra (U B1, B2 U^+, the
 // traceless anti-Hermitian projection) runs in FP32 on those sums: GB300's FP64 pipe is 1/64 of
 // its FP32 pipe, and FP64 algebra made the kernel 5x slower for an answer whose error is set by
-// the FP32 fields and block sums anyway. FP64 fields use FP64 throughout. F and G are written
+// the FP32 fields and block sums anyway. FP64 fields: k_force_fx below. F and G are written
 // in the canonical FP64 layout [t][z][y][x][mu][3][3].
-#include <type_traits>
+#include <algorithm>
 
 #include "dhop_kernel.cuh"
 #include "ff_arith.cuh"
+#include "fx_arith.cuh"
 
 namespace gdwf {
 
-// Threads per site: slice pairs (FP32, at most 128 for Ls <= 256) or padded slices (FP64; above 128
-// slices each thread takes several); sites per CTA fill 128 threads.
+// Threads per site: slice pairs (k_force) or padded slices (k_force_ff); sites per CTA fill 128 threads.
 inline int force_threads_per_site(int prec, int Ls) {
   const int n = prec == P64 ? ls_padded(Ls) : ls_half(Ls);
   return n < 128 ? n : 128;
@@ -111,16 +111,14 @@ __device__ __forceinline__ void force_site_algebra(int mu, int p, int first, int
   }
 }
 
-template <int P, bool C12>
+template <bool C12>
 __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, const char* chi, const char* Ue,
                                                const char* Uo, double* F, double* G, double coef, int nsg, int spc) {
-  using T = typename Store<P>::T;
-  using R = typename Store<P>::R;
-  using A = typename std::conditional<P == P64, double, float>::type;  // partial sums and link algebra
-  constexpr int LB = link_bytes(sizeof(T), C12);
-  constexpr int FLUSH = 8;  // FP32: slice pairs summed in FP32 before an FP64 sum across blocks
+  constexpr int P = P32;
+  using A = float;  // partial sums and link algebra
+  constexpr int FLUSH = 8;  // slice pairs summed in FP32 before an FP64 sum across blocks
   const int Lsh = ls_half(g.Ls);
-  const size_t site_bytes = (size_t)Lsh * 2 * 24 * sizeof(T);
+  const size_t site_bytes = (size_t)Lsh * 2 * 24 * sizeof(float);
   const size_t half_bytes = (size_t)g.N4h * site_bytes;
   // both parities of a block of sites run next to each other, so their shared neighbours are
   // still in L2 when the other parity reads them
@@ -128,7 +126,7 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
   const int first = (blockIdx.x >> 1) * spc;
   const int tid = threadIdx.x;
   const int site_local = tid / nsg;
-  const int t = tid - site_local * nsg;  // slice pair (FP32) or slice (FP64)
+  const int t = tid - site_local * nsg;  // slice pair
   const int nsites = min(spc, g.N4h - first);
   const bool active = site_local < nsites;
   const int i = first + (active ? site_local : 0);
@@ -156,61 +154,28 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
       const char* psi_f = psi + (1 - p) * half_bytes + site_offset(j, Lsh, site_bytes);
       const char* chi_f = chi + (1 - p) * half_bytes + site_offset(j, Lsh, site_bytes);
       A* dst = part + ((size_t)site_local * nsg + t) * FORCE_PART_STRIDE;
-      if constexpr (P == P64) {
-        double B[36];
 #pragma unroll
-        for (int k = 0; k < 36; ++k) B[k] = 0;
-        for (int sl5 = t; sl5 < 2 * Lsh; sl5 += nsg) {  // this thread's slices (one unless Ls > 128)
+      for (int term = 0; term < 2; ++term) {
+        float2 v[24], ha[12], hb[12];
+        load_pair<P, 0>(term == 0 ? psi_f : psi_x, t, Lsh, v);
+        if (term == 0) project2<-1>(mu, v, ha); else project2<+1>(mu, v, ha);
+        load_pair<P, 0>(term == 0 ? chi_x : chi_f, t, Lsh, v);
+        if (term == 0) project2<-1>(mu, v, hb); else project2<+1>(mu, v, hb);
 #pragma unroll
-          for (int term = 0; term < 2; ++term) {
-            double v[24], ha[12], hb[12];
-            load_lane64<0>(term == 0 ? psi_f : psi_x, sl5, Lsh, v);
-            if (term == 0) project<-1>(mu, v, ha); else project<+1>(mu, v, ha);
-            load_lane64<0>(term == 0 ? chi_x : chi_f, sl5, Lsh, v);
-            if (term == 0) project<-1>(mu, v, hb); else project<+1>(mu, v, hb);
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-            for (int a = 0; a < 3; ++a)
+          for (int b = 0; b < 3; ++b) {  // both slices of the pair, then their sum
+            float2 re = make_float2(0.f, 0.f), im = make_float2(0.f, 0.f);
 #pragma unroll
-              for (int b = 0; b < 3; ++b) {  // sum_h ha[h][a] conj(hb[h][b])
-                double re = B[term * 18 + (a * 3 + b) * 2], im = B[term * 18 + (a * 3 + b) * 2 + 1];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  const double xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
-                  const double yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
-                  re = fma(xr, yr, fma(xi, yi, re));
-                  im = fma(xi, yr, fma(-xr, yi, im));
-                }
-                B[term * 18 + (a * 3 + b) * 2] = re;
-                B[term * 18 + (a * 3 + b) * 2 + 1] = im;
-              }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 36; ++k) dst[k] = B[k];
-      } else {
-#pragma unroll
-        for (int term = 0; term < 2; ++term) {
-          float2 v[24], ha[12], hb[12];
-          load_pair<P, 0>(term == 0 ? psi_f : psi_x, t, Lsh, v);
-          if (term == 0) project2<-1>(mu, v, ha); else project2<+1>(mu, v, ha);
-          load_pair<P, 0>(term == 0 ? chi_x : chi_f, t, Lsh, v);
-          if (term == 0) project2<-1>(mu, v, hb); else project2<+1>(mu, v, hb);
-#pragma unroll
-          for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {  // both slices of the pair, then their sum
-              float2 re = make_float2(0.f, 0.f), im = make_float2(0.f, 0.f);
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const float2 xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
-                const float2 yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
-                re = ffma2(xr, yr, ffma2(xi, yi, re));
-                im = ffma2(xi, yr, ffma2(make_float2(-xr.x, -xr.y), yi, im));
-              }
-              dst[term * 18 + (a * 3 + b) * 2] = re.x + re.y;
-              dst[term * 18 + (a * 3 + b) * 2 + 1] = im.x + im.y;
+            for (int h = 0; h < 2; ++h) {
+              const float2 xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
+              const float2 yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
+              re = ffma2(xr, yr, ffma2(xi, yi, re));
+              im = ffma2(xi, yr, ffma2(make_float2(-xr.x, -xr.y), yi, im));
             }
-        }
+            dst[term * 18 + (a * 3 + b) * 2] = re.x + re.y;
+            dst[term * 18 + (a * 3 + b) * 2 + 1] = im.x + im.y;
+          }
       }
     }
     __syncthreads();
@@ -219,10 +184,7 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
       const int sl = task / 36, e = task - sl * 36;
       const A* src = part + (size_t)sl * nsg * FORCE_PART_STRIDE + e;
       A total;
-      if constexpr (P == P64) {
-        total = 0;
-        for (int k = 0; k < nsg; ++k) total += src[(size_t)k * FORCE_PART_STRIDE];
-      } else if (nsg <= FLUSH) {  // one block: FP32 throughout
+      if (nsg <= FLUSH) {  // one block: FP32 throughout
         total = 0.f;
         for (int k = 0; k < nsg; ++k) total += src[(size_t)k * FORCE_PART_STRIDE];
       } else {  // blocks of FLUSH pairs summed in FP64
@@ -427,6 +389,316 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
   }
 }
 
+// FP64 fields in block integers (fx_arith.cuh): with IEEE instructions the 192 FP64 operations per
+// (site, slice, direction) ran at 2 per SM and clock (16^4 x 12 force call 2.14 ms, 1.7 ms of it here).
+// Two threads (neighbouring lanes) per (site, slice), one per term: with own = chi(x) and nb = psi(x + mu)
+// for B1, own = psi(x) and nb = chi(x + mu) for B2, either forms C = sum_h (P nb)_h (x) (P own)_h^*
+// (B1 = C, B2 = C^+), the digits of the own spinor waiting in shared memory. The 9 complex sums are
+// exact 64-bit integers per slice (4 products each, < 2^62), aligned by a rounded shift to the
+// largest slice's exponent while they are added over the site's slices, and rounded to FP64 once. The
+// link algebra of all four directions follows at the end, in FP64, 36 entries per site (direction by
+// direction, with 36 of 128 threads at work between barriers: force call at 16^4 x 16 1612 us; with
+// FP64 products 2520 us; now 1288 us, of which M psi is 470 us). Integer instructions and the barriers
+// around the slice sums bound it now. A block of sites with a magnitude outside the integer range takes force_products_ieee
+// instead, for all its slices.
+constexpr int FORCE_FX_STRIDE = 19;  // 64-bit values per (slice, term): 18, odd so that stores spread over the banks
+constexpr int FORCE_FX_OWN = 25;     // digit pairs per thread of the own spinor: 24, odd for the same reason
+// Threads and sites per CTA at most (Ls > 32: one site). 256 threads, two CTAs per SM instead of four,
+// wait longer at the barriers: 1382 us.
+constexpr int FORCE_FX_THREADS = 128, FORCE_FX_SITES = 16;
+
+__device__ __noinline__ void force_products_ieee(const char* psi_x, const char* chi_x, const char* psi_f,
+                                                 const char* chi_f, int mu, int s, int Lsh, double* B) {
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    if (m != mu) continue;
+#pragma unroll
+    for (int term = 0; term < 2; ++term) {
+      double v[24], ha[12], hb[12];
+      load_lane64<0>(term == 0 ? psi_f : psi_x, s, Lsh, v);
+      if (term == 0) project<-1>(m, v, ha); else project<+1>(m, v, ha);
+      load_lane64<0>(term == 0 ? chi_x : chi_f, s, Lsh, v);
+      if (term == 0) project<-1>(m, v, hb); else project<+1>(m, v, hb);
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {  // sum_h ha[h][a] conj(hb[h][b])
+          double re = 0, im = 0;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const double xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
+            const double yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
+            re = fma(xr, yr, fma(xi, yi, re));
+            im = fma(xi, yr, fma(-xr, yi, im));
+          }
+          B[term * 18 + (a * 3 + b) * 2] = re;
+          B[term * 18 + (a * 3 + b) * 2 + 1] = im;
+        }
+    }
+  }
+}
+
+inline size_t force_fx_smem(int nsg, int spc) {
+  return (size_t)spc * 4 * 36 * 8 + (size_t)spc * nsg * (FORCE_FX_OWN * 8 + FORCE_FX_STRIDE * 8) + (size_t)spc * 8;
+}
+
+template <bool C12>
+__global__ void __maxnreg__(128) k_force_fx(const Geom g, const char* psi, const char* chi, const char* Ue,
+                                            const char* Uo, double* F, double* G, double coef, int nsg, int spc,
+                                            int sum_shift) {
+  const int Lsh = ls_half(g.Ls), Lsp = 2 * Lsh;
+  const size_t site_bytes = (size_t)Lsp * 24 * 8;
+  const size_t half_bytes = (size_t)g.N4h * site_bytes;
+  const size_t cs = chunk_stride(Lsh);
+  const int p = blockIdx.x & 1;
+  const int first = (blockIdx.x >> 1) * spc;
+  const int tid = threadIdx.x;
+  const int site_local = tid / nsg;
+  const int ts = tid - site_local * nsg;
+  const int s = ts >> 1, t = ts & 1;  // slice, term
+  const int nsites = min(spc, g.N4h - first);
+  const int i = first + min(site_local, nsites - 1);  // threads past the end repeat the last site
+  int c[4];
+  cb_coords(g, i, p, c);
+
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* bsum = reinterpret_cast<double*>(smem_raw);                               // [spc][mu][36]
+  int2* own_sm = reinterpret_cast<int2*>(bsum + (size_t)spc * 4 * 36);              // [thread][real]
+  long long* part = reinterpret_cast<long long*>(own_sm + (size_t)FORCE_FX_OWN * nsg * spc);  // [spc][slice][term][19]
+  int* e_sm = reinterpret_cast<int*>(part + (size_t)spc * nsg * FORCE_FX_STRIDE);   // [spc][term]
+  if (ts < 2) e_sm[2 * site_local + ts] = 0;
+  int nf[4], pf[4];  // forward neighbours (the phases enter with the link algebra)
+#pragma unroll
+  for (int m = 0; m < 4; ++m) nf[m] = cb_neighbour(g, i, c, m, true, pf[m]);
+
+  const size_t xo = p * half_bytes + site_offset(i, Lsh, site_bytes);
+  const char* own_field = t == 0 ? chi : psi;
+  const char* nb_field = t == 0 ? psi : chi;
+  bool bad = false;
+  // exponent field of a block's largest real, at least FX_LO; flags what does not fit
+  auto block_exponent = [&](const double* v) {
+    uint32_t emax = fx_max_hi<24>(v) & 0x7ff00000u;
+    if (emax < ((uint32_t)FX_LO << 20)) {
+      if (!fx_all_zero<24>(v)) bad = true;
+      emax = (uint32_t)FX_LO << 20;
+    }
+    if (emax > ((uint32_t)FX_HI << 20)) {
+      bad = true;
+      emax = (uint32_t)FX_HI << 20;
+    }
+    return emax;
+  };
+  int2* own = own_sm + tid * FORCE_FX_OWN;
+  int e_own;
+  {
+    double v[24];
+    load_lane64<0>(own_field + xo, s, Lsh, v);
+    const uint32_t emax = block_exponent(v);
+    e_own = (int)(emax >> 20);
+#pragma unroll
+    for (int r = 0; r < 24; ++r) {
+      int y1, y0;
+      const int hi = __double2hiint(v[r]), sg = (hi >> 31) | 1;
+      fx_magnitude<8>((uint32_t)hi, (uint32_t)__double2loint(v[r]), emax, y1, y0);
+      own[r] = make_int2(y1 * sg, y0 * sg);
+    }
+  }
+  __syncthreads();
+
+#pragma unroll 1
+  for (int mu = 0; mu < 4; ++mu) {
+    const int j = mu == 0 ? nf[0] : mu == 1 ? nf[1] : mu == 2 ? nf[2] : nf[3];
+    const size_t jo = (1 - p) * half_bytes + site_offset(j, Lsh, site_bytes);
+    // h_k = psi_k +- (1 or i) psi_{p_k}, p = (3, 2) for x and y, (2, 3) for z and t: signs as a nibble
+    // {k=0 re, k=0 im, k=1 re, k=1 im} (bit set: subtract) for (1 + gamma), complemented for (1 - gamma)
+    const bool im_form = (mu & 1) == 0;  // i psi: real and imaginary parts trade places
+    const uint32_t neg = ((0x063Au >> (4 * mu)) & 15u) ^ (t ? 0u : 15u);
+    int n1[12], n0[12];  // digits of the projected neighbour spinor
+    int e_sum;
+    {
+      double v[24];  // the upper spins, then their partners (second spin of k, parts exchanged if im_form)
+      const char* nb = nb_field + jo + (size_t)s * 8;
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) {
+          const char* lo = nb + (mu < 2 ? 18 - 6 * k : 12 + 6 * k) * cs + 2 * cc * cs;
+          v[6 * k + 2 * cc] = __ldg(reinterpret_cast<const double*>(nb + (6 * k + 2 * cc) * cs));
+          v[6 * k + 2 * cc + 1] = __ldg(reinterpret_cast<const double*>(nb + (6 * k + 2 * cc + 1) * cs));
+          v[12 + 6 * k + 2 * cc] = __ldg(reinterpret_cast<const double*>(lo + (im_form ? cs : 0)));
+          v[12 + 6 * k + 2 * cc + 1] = __ldg(reinterpret_cast<const double*>(lo + (im_form ? 0 : cs)));
+        }
+      const uint32_t emax = block_exponent(v);
+      e_sum = (int)(emax >> 20) + e_own;
+#pragma unroll
+      for (int r = 0; r < 12; ++r) {
+        const int fl = -(int)((neg >> (2 * (r / 6) + (r & 1))) & 1u);
+        const int uh = __double2hiint(v[r]), lh = __double2hiint(v[12 + r]);
+        int u1, u0, l1, l0;
+        fx_magnitude<8>((uint32_t)uh, (uint32_t)__double2loint(v[r]), emax, u1, u0);
+        fx_magnitude<8>((uint32_t)lh, (uint32_t)__double2loint(v[12 + r]), emax, l1, l0);
+        const int su = (uh >> 31) | 1, sl = ((lh >> 31) ^ fl) | 1;
+        n1[r] = l1 * sl + u1 * su;
+        n0[r] = l0 * sl + u0 * su;
+      }
+    }
+    int* emax = e_sm + 2 * site_local + t;  // largest exponent of the site's slices in this term
+    atomicMax(emax, e_sum);
+    long long C[18];
+    // the nine complex sums, 2^(e_sum - 2102) each; where the own projection reads its second spins
+    const int2* partner[4];
+    int psign[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const int k = h >> 1, im = h & 1;
+      partner[h] = own + (mu < 2 ? 18 - 6 * k : 12 + 6 * k) + (im_form ? 1 - im : im);
+      psign[h] = (neg >> h) & 1u ? -1 : 1;
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      // digits of the projected own spinor, colour b: [h][re, im]
+      int o1[4], o0[4];
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int2 u = own[6 * (h >> 1) + 2 * b + (h & 1)];
+        const int2 l = partner[h][2 * b];
+        o1[h] = l.x * psign[h] + u.x;
+        o0[h] = l.y * psign[h] + u.y;
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        long long hr = 0, hi = 0, cr = 1ll << 27, ci = 1ll << 27;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int xr1 = n1[6 * k + 2 * a], xr0 = n0[6 * k + 2 * a];
+          const int xi1 = n1[6 * k + 2 * a + 1], xi0 = n0[6 * k + 2 * a + 1];
+          const int yr1 = o1[2 * k], yr0 = o0[2 * k], yi1 = o1[2 * k + 1], yi0 = o0[2 * k + 1];
+          const int zi1 = -yi1, zi0 = -yi0;
+          hr += (long long)xr1 * yr1;
+          cr += (long long)xr1 * yr0;
+          cr += (long long)xr0 * yr1;
+          hr += (long long)xi1 * yi1;
+          cr += (long long)xi1 * yi0;
+          cr += (long long)xi0 * yi1;
+          hi += (long long)xi1 * yr1;
+          ci += (long long)xi1 * yr0;
+          ci += (long long)xi0 * yr1;
+          hi += (long long)xr1 * zi1;
+          ci += (long long)xr1 * zi0;
+          ci += (long long)xr0 * zi1;
+        }
+        C[(a * 3 + b) * 2] = hr + (cr >> 28);
+        C[(a * 3 + b) * 2 + 1] = hi + (ci >> 28);
+      }
+    }
+    const bool any_bad = __syncthreads_or(bad) != 0;  // also: every exponent is in e_sm
+    long long* dst = part + (size_t)tid * FORCE_FX_STRIDE;
+    if (!any_bad) {
+      // to the site's largest exponent, and sum_shift bits further for the sum over the slices
+      const int d = *emax - e_sum + sum_shift;
+      const long long half = d > 0 && d < 64 ? 1ll << (d - 1) : 0;
+#pragma unroll
+      for (int k = 0; k < 18; ++k) dst[k] = d < 64 ? (C[k] + half) >> d : 0;
+    } else if (t == 0) {
+      double B[36];
+      force_products_ieee(psi + xo, chi + xo, psi + jo, chi + jo, mu, s, Lsh, B);
+      double* both = reinterpret_cast<double*>(dst);  // both lanes' slots
+      for (int k = 0; k < 36; ++k) both[k] = B[k];
+    }
+    __syncthreads();
+    // sums over the site's slices, one (site, entry) per task
+    for (int task = tid; task < nsites * 36; task += blockDim.x) {
+      const int sl = task / 36, e = task - sl * 36, term = e / 18, k = e - term * 18;
+      double v = 0;
+      if (!any_bad) {
+        // B2 = C^+: entry (a, b) from (b, a), imaginary part negated
+        const int ab = k >> 1, a = ab / 3, b = ab - a * 3;
+        const int kk = term ? (b * 3 + a) * 2 + (k & 1) : k;
+        const long long* src = part + ((size_t)sl * nsg + term) * FORCE_FX_STRIDE + kk;
+        long long tot = 0;
+        for (int q = 0; q < Lsp; ++q) tot += src[q * (2 * FORCE_FX_STRIDE)];
+        v = (double)tot;
+        const int ex = e_sm[2 * sl + term] + sum_shift - 2102;
+        if (tot != 0) v = __hiloint2double(__double2hiint(v) + (ex << 20), __double2loint(v));
+        if (term && (k & 1)) v = -v;
+      } else {
+        const double* src = reinterpret_cast<const double*>(part + (size_t)sl * nsg * FORCE_FX_STRIDE) + e;
+        for (int q = 0; q < Lsp; ++q) v += src[q * (2 * FORCE_FX_STRIDE)];
+      }
+      bsum[((size_t)sl * 4 + mu) * 36 + e] = v;
+    }
+    __syncthreads();  // shared memory is reused by the next direction
+    if (ts < 2) e_sm[2 * site_local + ts] = 0;
+    __syncthreads();
+  }
+
+  // ---- link algebra (see force_site_algebra), links and Y in the own spinors' place; tasks (site, mu, a, b)
+  constexpr int LB = link_bytes(8, C12);
+  double* usm = reinterpret_cast<double*>(own_sm);  // [spc][mu][18]
+  double* ysm = usm + (size_t)spc * 4 * 18;        // [spc][mu][18]
+  for (int task = tid; task < nsites * 4; task += blockDim.x) {
+    double u[18];
+    load_link<P64, C12>((p ? Uo : Ue) + ((size_t)first * 4 + task) * LB, u);
+#pragma unroll
+    for (int k = 0; k < 18; ++k) usm[(size_t)task * 18 + k] = u[k];
+  }
+  __syncthreads();
+  // site of the CTA and direction of a task: canonical index of the link and its boundary phase
+  auto link_of = [&](int task, size_t& out, double& ph) {
+    const int sl = task / 36, mu = (task - sl * 36) / 9;
+    int x[4];
+    cb_coords(g, first + sl, p, x);
+    const long lex = x[0] + (long)g.L[0] * (x[1] + (long)g.L[1] * (x[2] + (long)g.L[2] * x[3]));
+    const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
+    const int L = mu == 0 ? g.L[0] : mu == 1 ? g.L[1] : mu == 2 ? g.L[2] : g.L[3];
+    const int bc = mu == 0 ? g.bc[0] : mu == 1 ? g.bc[1] : mu == 2 ? g.bc[2] : g.bc[3];
+    out = ((size_t)lex * 4 + mu) * 18;
+    ph = xm == L - 1 && bc < 0 ? -coef : coef;  // F and G are linear in the boundary phase and coef
+  };
+  for (int task = tid; task < nsites * 36; task += blockDim.x) {
+    const int link = task / 9, ab = task - link * 9, a = ab / 3, b = ab - a * 3;
+    size_t out;
+    double ph;
+    link_of(task, out, ph);
+    const double* B1 = bsum + (size_t)link * 36;
+    const double* B2 = B1 + 18;
+    const double* ur = usm + (size_t)link * 18;
+    double yr = 0, yi = 0;  // -U B1 + B2 U^+
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double ar = ur[(a * 3 + k) * 2], ai = ur[(a * 3 + k) * 2 + 1];
+      const double br = B1[(k * 3 + b) * 2], bi = B1[(k * 3 + b) * 2 + 1];
+      yr = fma(-ar, br, fma(ai, bi, yr));
+      yi = fma(-ar, bi, fma(-ai, br, yi));
+      const double cr = B2[(a * 3 + k) * 2], ci = B2[(a * 3 + k) * 2 + 1];
+      const double dr = ur[(b * 3 + k) * 2], di = ur[(b * 3 + k) * 2 + 1];  // (U^+)[k][b] = conj(U[b][k])
+      yr = fma(cr, dr, fma(ci, di, yr));
+      yi = fma(ci, dr, fma(-cr, di, yi));
+    }
+    ysm[(size_t)link * 18 + ab * 2] = ph * yr;
+    ysm[(size_t)link * 18 + ab * 2 + 1] = ph * yi;
+    if (G) {
+      G[out + ab * 2] = -ph * (B1[(b * 3 + a) * 2] + B2[ab * 2]);
+      G[out + ab * 2 + 1] = -ph * (B2[ab * 2 + 1] - B1[(b * 3 + a) * 2 + 1]);
+    }
+  }
+  __syncthreads();
+  if (F) {
+    for (int task = tid; task < nsites * 36; task += blockDim.x) {
+      const int link = task / 9, ab = task - link * 9, a = ab / 3, b = ab - a * 3;
+      size_t out;
+      double ph;
+      link_of(task, out, ph);
+      const double* Y = ysm + (size_t)link * 18;
+      const double re = 0.5 * (Y[(b * 3 + a) * 2] - Y[(a * 3 + b) * 2]);
+      double im = -0.5 * (Y[(a * 3 + b) * 2 + 1] + Y[(b * 3 + a) * 2 + 1]);
+      if (a == b) im += (Y[1] + Y[9] + Y[17]) * (1.0 / 3.0);
+      F[out + ab * 2] = re;
+      F[out + ab * 2 + 1] = im;
+    }
+  }
+}
+
 // FP64 fields in float-float arithmetic (the handle's FP64 arithmetic set to float-float): the
 // per-slice products in pairs of FP32 numbers, the slice sums in float-float, then the site's
 // sums rounded to FP64 for the (per 4D site, cheap) link algebra. One thread per (site, slice)
@@ -536,11 +808,6 @@ cudaError_t launch_force(int prec, bool c12, const Geom& g, const void* psi, con
   const char* ch = static_cast<const char*>(chi);
   const char* e = static_cast<const char*>(Ue);
   const char* o = static_cast<const char*>(Uo);
-#define FK(P_)                                                                                 \
-  if (c12)                                                                                     \
-    k_force<P_, true><<<grid, threads, smem, st>>>(g, ps, ch, e, o, F, G, coef, nsg, spc);    \
-  else                                                                                         \
-    k_force<P_, false><<<grid, threads, smem, st>>>(g, ps, ch, e, o, F, G, coef, nsg, spc);
   if (prec == P64 && float_float) {
     if (c12)
       k_force_ff<true><<<grid, threads, smem, st>>>(g, ps, ch, e, o, F, G, coef, nsg, spc);
@@ -549,6 +816,21 @@ cudaError_t launch_force(int prec, bool c12, const Geom& g, const void* psi, con
     return cudaGetLastError();
   }
   const int Lsh = ls_half(g.Ls);
+  if (prec == P64) {
+    const int n2 = 2 * ls_padded(g.Ls);  // two threads per slice
+    const int s2 = std::max(1, std::min(FORCE_FX_THREADS / n2, FORCE_FX_SITES));
+    int shift = 0;
+    while ((1 << shift) < g.Ls) ++shift;
+    const size_t sm = force_fx_smem(n2, s2);
+    const dim3 gr((unsigned)(2 * ((g.N4h + s2 - 1) / s2)));
+    auto kern = c12 ? k_force_fx<true> : k_force_fx<false>;
+    if (sm > 48 * 1024) {
+      cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (err != cudaSuccess) return err;
+    }
+    kern<<<gr, n2 * s2, sm, st>>>(g, ps, ch, e, o, F, G, coef, n2, s2, shift);
+    return cudaGetLastError();
+  }
   if (prec == P32 && (Lsh == 8 || Lsh == 16)) {
     // CTAs of 64 threads for 8 pairs per site (8 sites; measured 108.2 us against 109.5 us with
     // 128 threads at 16^4 x 16, the same warps per SM and a finer last wave), 128 for 16 pairs
@@ -565,12 +847,11 @@ cudaError_t launch_force(int prec, bool c12, const Geom& g, const void* psi, con
 #undef FR
     return cudaGetLastError();
   }
-  switch (prec) {
-    case P64: FK(P64) break;
-    case P32: FK(P32) break;
-    default: return cudaErrorInvalidValue;
-  }
-#undef FK
+  if (prec != P32) return cudaErrorInvalidValue;
+  if (c12)
+    k_force<true><<<grid, threads, smem, st>>>(g, ps, ch, e, o, F, G, coef, nsg, spc);
+  else
+    k_force<false><<<grid, threads, smem, st>>>(g, ps, ch, e, o, F, G, coef, nsg, spc);
   return cudaGetLastError();
 }
 
