@@ -204,10 +204,11 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
   }
 }
 
-// FP32 fields with 8 or 16 slice pairs per site (Ls 15-16, 31-32; the static shared memory of
-// fewer pairs per site, i.e. more sites per CTA, would pass 48 KB): a site's
-// threads are LSH consecutive lanes of one warp, so the sums over its slices run in registers and
-// every synchronisation is within a warp.
+// FP32 fields with 3 to 16 slice pairs per site: a site's threads are LG consecutive lanes of one warp
+// (4, 8 or 16; FULL: one per pair, otherwise the lanes past the last pair add zeros), so the sums over
+// its slices run in registers and every synchronisation is within a warp. Lanes left idle cost less than
+// k_force's sums through shared memory: force call at 16^4 with Ls = 10 / 12 / 24, k_force and this:
+// 265 / 244 / 395 and 211 / 215 / 351 us. (With 2 lanes, the 32 sites of a CTA would pass 48 KB of static shared memory.)
 //   - Each field is read once as the own site's spinor: the B1 products of all four directions
 //     first (own chi(x) held in registers, psi(x + mu) loaded per direction), then the B2 products
 //     (own psi(x) held, chi(x + mu) loaded): 10 spinor loads per (site, pair) instead of 16.
@@ -218,11 +219,11 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
 //   - The link algebra of the site's four links (36 entries) is spread over the same lanes.
 // Rounding: the products of a slice pair and the sums over at most 16 pairs are FP32, as in the
 // general kernel (which flushes to FP64 after 8 pairs; here 16 pairs at most are summed in FP32).
-template <int LSH, int THREADS = 128>
+template <int LG, int THREADS>
 struct ForceRegGeom {
-  static constexpr int SPC = THREADS / LSH;                         // sites per CTA
-  static constexpr int PER_LANE = (18 + LSH - 1) / LSH;              // sum entries per lane after reduce-scatter
-  static constexpr int NPAD = PER_LANE * LSH;                         // 18 reals padded to a multiple of LSH
+  static constexpr int SPC = THREADS / LG;               // sites per CTA
+  static constexpr int PER_LANE = (18 + LG - 1) / LG;    // sum entries per lane after reduce-scatter
+  static constexpr int NPAD = PER_LANE * LG;             // 18 reals padded to a multiple of LG
   // B1 B2 per mu, U per mu, Y per mu, padded so that the sites of a warp fall on different banks:
   // 299 floats give the fewest conflicts of the strides 289-329 over the partial-sum stores and the
   // link algebra's reads of 8-lane sites (53 extra wavefronts per warp against 116 at 289, by
@@ -248,20 +249,23 @@ __device__ __forceinline__ void reduce_scatter(float (&v)[N], int lane_in_site) 
 // The own spinor of a term goes through shared memory and is read back per direction (128
 // registers, 4 CTAs per SM): holding it in 48 registers instead needed 168 registers, 3 CTAs per
 // SM and some spills, and measured 136 us against 111 us at 16^4 x 16.
-template <bool C12, int LSH, int THREADS = 128>
+template <bool C12, int LG, bool FULL, int THREADS>
 __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom g, const char* psi, const char* chi,
                                                                       const char* Ue, const char* Uo, double* F,
                                                                       double* G, double coef) {
-  using GG = ForceRegGeom<LSH, THREADS>;
+  using GG = ForceRegGeom<LG, THREADS>;
   constexpr int LB = link_bytes(4, C12);
   constexpr int SPC = GG::SPC, NPAD = GG::NPAD, PER_LANE = GG::PER_LANE;
-  const size_t site_bytes = (size_t)LSH * 2 * 24 * 4;
+  constexpr int LSH = FULL ? LG : 0;
+  const int Lsh = FULL ? LG : ls_half(g.Ls);
+  const size_t site_bytes = (size_t)Lsh * 2 * 24 * 4;
   const size_t half_bytes = (size_t)g.N4h * site_bytes;
   const int p = blockIdx.x & 1;
   const int first = (blockIdx.x >> 1) * SPC;
   const int tid = threadIdx.x;
-  const int site_local = tid / LSH;
-  const int q = tid - site_local * LSH;  // slice pair, and the lane's place in its site's group
+  const int site_local = tid / LG;
+  const int q = tid - site_local * LG;  // slice pair, and the lane's place in its site's group
+  const bool has_pair = FULL || q < Lsh;
   const bool active = first + site_local < g.N4h;
   const int i = active ? first + site_local : first;  // inactive lanes compute a valid site, store nothing
   int c[4];
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
   float* ys = us + 4 * 18;              // [mu][18]
 
   // the site's four links U_mu(x), one per lane (and the third row rebuilt for 12-real links)
-  for (int mu = q; mu < 4; mu += LSH) {
+  for (int mu = q; mu < 4; mu += LG) {
     float ur[18];
     load_link<P32, C12>((p ? Uo : Ue) + ((size_t)i * 4 + mu) * LB, ur);
 #pragma unroll
@@ -290,52 +294,54 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
   for (int term = 0; term < 2; ++term) {
     // term 0: B1 = sum psi(x+mu) (x) [(1 - gamma) chi(x)]^+  (own chi, projector sign -1)
     // term 1: B2 = sum psi(x) (x) [(1 + gamma) chi(x+mu)]^+  (own psi, projector sign +1)
-    {
-      const char* ob = (term == 0 ? chi : psi) + p * half_bytes + site_offset(i, LSH, site_bytes) + (size_t)q * 16;
+    if (has_pair) {
+      const char* ob = (term == 0 ? chi : psi) + p * half_bytes + site_offset(i, Lsh, site_bytes) + (size_t)q * 16;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) own_sm[k][tid] = __ldg(reinterpret_cast<const float4*>(ob + k * chunk_stride(LSH)));
+      for (int k = 0; k < 12; ++k) own_sm[k][tid] = __ldg(reinterpret_cast<const float4*>(ob + k * chunk_stride(Lsh)));
     }
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-      float2 v[24], ha[12], hb[12];
-      load_pair<P32, LSH>((term == 0 ? psi : chi) + (1 - p) * half_bytes + site_offset(nbr[mu], LSH, site_bytes), q,
-                          LSH, v);
-      {
-        float2 own[24];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          const float4 t = own_sm[k][tid];
-          own[2 * k] = make_float2(t.x, t.y);
-          own[2 * k + 1] = make_float2(t.z, t.w);
-        }
-        if (term == 0)
-          project2<-1>(mu, own, hb);
-        else
-          project2<+1>(mu, own, ha);
-      }
-      if (term == 0)
-        project2<-1>(mu, v, ha);
-      else
-        project2<+1>(mu, v, hb);
       float s[NPAD];
 #pragma unroll
-      for (int k = 18; k < NPAD; ++k) s[k] = 0.f;
+      for (int k = 0; k < NPAD; ++k) s[k] = 0.f;
+      if (has_pair) {
+        float2 v[24], ha[12], hb[12];
+        load_pair<P32, LSH>((term == 0 ? psi : chi) + (1 - p) * half_bytes + site_offset(nbr[mu], Lsh, site_bytes), q,
+                            Lsh, v);
+        {
+          float2 own[24];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {  // sum_h ha[h][a] conj(hb[h][b]), both slices of the pair
-          float2 re = make_float2(0.f, 0.f), im = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const float2 xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
-            const float2 yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
-            re = ffma2(xr, yr, ffma2(xi, yi, re));
-            im = ffma2(xi, yr, ffma2(make_float2(-xr.x, -xr.y), yi, im));
+          for (int k = 0; k < 12; ++k) {
+            const float4 t = own_sm[k][tid];
+            own[2 * k] = make_float2(t.x, t.y);
+            own[2 * k + 1] = make_float2(t.z, t.w);
           }
-          s[(a * 3 + b) * 2] = re.x + re.y;
-          s[(a * 3 + b) * 2 + 1] = im.x + im.y;
+          if (term == 0)
+            project2<-1>(mu, own, hb);
+          else
+            project2<+1>(mu, own, ha);
         }
-      reduce_scatter<NPAD, LSH>(s, q);
+        if (term == 0)
+          project2<-1>(mu, v, ha);
+        else
+          project2<+1>(mu, v, hb);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {  // sum_h ha[h][a] conj(hb[h][b]), both slices of the pair
+            float2 re = make_float2(0.f, 0.f), im = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float2 xr = ha[(h * 3 + a) * 2], xi = ha[(h * 3 + a) * 2 + 1];
+              const float2 yr = hb[(h * 3 + b) * 2], yi = hb[(h * 3 + b) * 2 + 1];
+              re = ffma2(xr, yr, ffma2(xi, yi, re));
+              im = ffma2(xi, yr, ffma2(make_float2(-xr.x, -xr.y), yi, im));
+            }
+            s[(a * 3 + b) * 2] = re.x + re.y;
+            s[(a * 3 + b) * 2 + 1] = im.x + im.y;
+          }
+      }
+      reduce_scatter<NPAD, LG>(s, q);
 #pragma unroll
       for (int k = 0; k < PER_LANE; ++k) {
         const int e = q * PER_LANE + k;
@@ -347,7 +353,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
   // link algebra, one (mu, a, b) entry per task over the site's lanes:
   //   G[a][b] = -phase (conj(B1[b][a]) + B2[a][b]),  Y = phase (-U B1 + B2 U^+)
   const long lex = c[0] + (long)g.L[0] * (c[1] + (long)g.L[1] * (c[2] + (long)g.L[2] * c[3]));
-  for (int task = q; task < 36; task += LSH) {
+  for (int task = q; task < 36; task += LG) {
     const int mu = task / 9, ab = task - mu * 9, a = ab / 3, b = ab - a * 3;
     const int ph = mu == 0 ? phs[0] : mu == 1 ? phs[1] : mu == 2 ? phs[2] : phs[3];
     const float phd = (float)(coef * (double)ph);
@@ -377,7 +383,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
   __syncwarp();
   // F = -TA(Y): TA(Y)[a][b] = (Y[a][b] - conj(Y[b][a]))/2 - delta_ab tr(Y - Y^+)/6
   if (F && active) {
-    for (int task = q; task < 36; task += LSH) {
+    for (int task = q; task < 36; task += LG) {
       const int mu = task / 9, ab = task - mu * 9, a = ab / 3, b = ab - a * 3;
       const float* Y = ys + mu * 18;
       const float trim = Y[1] + Y[9] + Y[17];  // Im tr Y; tr(Y - Y^+) = 2 i Im tr Y
@@ -831,19 +837,18 @@ cudaError_t launch_force(int prec, bool c12, const Geom& g, const void* psi, con
     kern<<<gr, n2 * s2, sm, st>>>(g, ps, ch, e, o, F, G, coef, n2, s2, shift);
     return cudaGetLastError();
   }
-  if (prec == P32 && (Lsh == 8 || Lsh == 16)) {
-    // CTAs of 64 threads for 8 pairs per site (8 sites; measured 108.2 us against 109.5 us with
-    // 128 threads at 16^4 x 16, the same warps per SM and a finer last wave), 128 for 16 pairs
+  if (prec == P32 && Lsh >= 3 && Lsh <= 16) {
+    // CTAs of 64 threads for up to 8 pairs per site (8 or 16 sites; measured 108.2 us against 109.5 us
+    // with 128 threads at 16^4 x 16, the same warps per SM and a finer last wave), 128 above
 #define FR(L_, T_)                                                                                       \
   {                                                                                                      \
     constexpr int spc = ForceRegGeom<L_, T_>::SPC;                                                       \
     const dim3 gr((unsigned)(2 * ((g.N4h + spc - 1) / spc)));                                            \
-    if (c12)                                                                                             \
-      k_force_reg<true, L_, T_><<<gr, T_, 0, st>>>(g, ps, ch, e, o, F, G, coef);                         \
-    else                                                                                                 \
-      k_force_reg<false, L_, T_><<<gr, T_, 0, st>>>(g, ps, ch, e, o, F, G, coef);                        \
+    auto kern = Lsh == L_ ? (c12 ? k_force_reg<true, L_, true, T_> : k_force_reg<false, L_, true, T_>)    \
+                          : (c12 ? k_force_reg<true, L_, false, T_> : k_force_reg<false, L_, false, T_>); \
+    kern<<<gr, T_, 0, st>>>(g, ps, ch, e, o, F, G, coef);                                                \
   }
-    if (Lsh == 8) FR(8, 64) else FR(16, 128)
+    if (Lsh <= 4) FR(4, 64) else if (Lsh <= 8) FR(8, 64) else FR(16, 128)
 #undef FR
     return cudaGetLastError();
   }
