@@ -1017,7 +1017,8 @@ cudaError_t launch_pack_gauge_fx(bool c12, const Geom& g, const double* canon, v
 // Threads per site: slice pairs (packed kernels) or padded slices (FP64).
 inline int dhop_threads_per_site(int prec, int Ls) { return prec == P64 ? ls_padded(Ls) : ls_half(Ls); }
 
-// FP64 kernels: Ls values with a compile-time specialisation; any other Ls runs the generic kernel (LSC = 0).
+// Float-float kernel: Ls values with a compile-time specialisation; any other Ls runs the generic kernel
+// (LSC = 0).
 #define DWF_LS_SPECIALISATIONS(M) M(8) M(12) M(16)
 inline bool dhop_ls_specialised(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 

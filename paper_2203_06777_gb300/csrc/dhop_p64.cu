@@ -446,11 +446,12 @@ size_t dhop_fx_smem_bytes(int sites_per_cta, int Ls, bool post) {
 template <>
 cudaError_t launch_dhop<P64>(const DhopArgs& a, bool dag, bool c12, int threads, int blocks, size_t smem,
                              cudaStream_t stream) {
-  switch (a.g.Ls) {
-#define DWF_CASE(L_) \
-  case L_:           \
-    return launch_fx<L_>(a, dag, c12, threads, blocks, smem, stream);
-    DWF_LS_SPECIALISATIONS(DWF_CASE)
+  // the even extents of the packed kernels (Ls / 2 pairs); any other Ls runs the generic kernel
+  switch (a.g.Ls & 1 ? 0 : a.g.Ls / 2) {
+#define DWF_CASE(N_) \
+  case N_:           \
+    return launch_fx<2 * N_>(a, dag, c12, threads, blocks, smem, stream);
+    DWF_PAIR_SPECIALISATIONS(DWF_CASE)
 #undef DWF_CASE
     default:
       return launch_fx<0>(a, dag, c12, threads, blocks, smem, stream);
