@@ -213,6 +213,10 @@ int grid_dwf_cg(grid_dwf_t* h, const void* b, void* x, double tol, int maxiter, 
  * scratch. Under U -> exp(eps A) U with A in su(3): dS/deps = sum Re tr(A^+ F). *S_out on host. */
 int grid_dwf_force(grid_dwf_t* h, int precision, const void* psi, void* chi, double* F, double* G, double* S_out);
 
+/* The contraction of grid_dwf_force alone, for a caller that holds chi = M psi already (full fields in the
+ * device layout; both only read): F and G (either may be NULL) as there. Asynchronous. */
+int grid_dwf_force_contract(grid_dwf_t* h, int precision, const void* psi, const void* chi, double* F, double* G);
+
 /* Two-flavour pseudofermion action S = phi^+ (Mpc^+ Mpc)^-1 phi and its link derivative: the
  * Schur normal operator above as it enters hybrid Monte Carlo, differentiated through the solve.
  * The paper names no action; this is the next step after the operator, its solver and the force

@@ -1108,6 +1108,26 @@ int grid_dwf_cg(grid_dwf_t* h, const void* b, void* x, double tol, int maxiter, 
   return finish(h, "cg");
 }
 
+int grid_dwf_force_contract(grid_dwf_t* h, int precision, const void* psi, const void* chi, double* F, double* G) {
+  const NvtxRange nvtx_("grid_dwf_force_contract");
+  if (!h) return GRID_DWF_ERR_INVALID_ARG;
+  if (precision != GRID_DWF_FP64 && precision != GRID_DWF_FP32)
+    return fail(h, GRID_DWF_ERR_INVALID_ARG, "force_contract: precision must be FP64 or FP32");
+  RET(check_ptr(h, psi, "psi"));
+  RET(check_ptr(h, chi, "chi"));
+  const size_t fb = subset_bytes(h, precision, GRID_DWF_FULL);
+  const size_t gb = (size_t)h->g.N4h * 2 * 4 * 18 * sizeof(double);
+  for (double* out : {F, G})
+    if (out && (overlap(out, gb, psi, fb) || overlap(out, gb, chi, fb)))
+      return fail(h, GRID_DWF_ERR_ALIAS, "force_contract: output overlaps an input");
+  RET(ensure_gauge(h, precision));
+  if (F || G)
+    CK(launch_force(precision, h->c12, h->g, psi, chi, h->gauge[precision][0], h->gauge[precision][1], F, G, 1.0,
+                    h->fp64_arith == GRID_DWF_FP64_ARITH_FLOAT_FLOAT, h->stream),
+       "force_contract");
+  return finish(h, "force_contract");
+}
+
 int grid_dwf_force(grid_dwf_t* h, int precision, const void* psi, void* chi, double* F, double* G, double* S_out) {
   const NvtxRange nvtx_("grid_dwf_force");
   if (!h) return GRID_DWF_ERR_INVALID_ARG;

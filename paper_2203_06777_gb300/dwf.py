@@ -115,6 +115,7 @@ def load(build: bool = True):
             "grid_dwf_inner": [vp, i, i, vp, vp, dp],
             "grid_dwf_cg": [vp, vp, vp, d, i, i, ctypes.POINTER(_CgStats)],
             "grid_dwf_force": [vp, i, vp, vp, vp, vp, dp],
+            "grid_dwf_force_contract": [vp, i, vp, vp, vp, vp],
             "grid_dwf_pf_force": [vp, vp, vp, d, i, i, i, vp, vp, dp, ctypes.POINTER(_CgStats)],
             "grid_dwf_pipe_peak": [i, vp, dp],
             "grid_dwf_face_bytes": [vp, i, ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(ctypes.c_size_t)],
@@ -286,7 +287,8 @@ class GridDWF:
                 raise ValueError("unpacking a half field needs subset=EVEN or subset=ODD")
             subset = FULL
         if out is None:
-            out = torch.zeros(self.canonical_shape(), dtype=torch.complex128, device=self.device)
+            alloc = torch.empty if subset == FULL else torch.zeros  # a full field writes every site
+            out = alloc(self.canonical_shape(), dtype=torch.complex128, device=self.device)
         self._call("grid_dwf_unpack", prec, subset, _ptr(f), _ptr(out))
         return out
 
@@ -404,6 +406,17 @@ class GridDWF:
         self._call("grid_dwf_force", prec, _ptr(psi_field), _ptr(chi), _ptr(F), _ptr(G), ctypes.byref(S))
         return S.value, F, G
 
+    def force_contract(self, psi_field: torch.Tensor, chi: torch.Tensor, want_F=True, want_G=True):
+        """The F and G of :meth:`force` for chi = M psi held already (no operator application)."""
+        prec = self._check_field(psi_field)
+        if self._check_field(chi) != prec or chi.numel() != psi_field.numel() or self._subset_of(chi) != FULL:
+            raise ValueError("force_contract needs two full fields of one precision")
+        lx, ly, lz, lt = self.dims
+        shape = (lt, lz, ly, lx, 4, 3, 3)
+        F = torch.empty(shape, dtype=torch.complex128, device=self.device) if want_F else None
+        G = torch.empty(shape, dtype=torch.complex128, device=self.device) if want_G else None
+        self._call("grid_dwf_force_contract", prec, _ptr(psi_field), _ptr(chi), _ptr(F), _ptr(G))
+        return F, G
 
     def pf_force(self, phi: torch.Tensor, x: torch.Tensor | None = None, tol=1e-10, maxiter=10000, mode=CG_FP64,
                  precision=FP64, want_F=True, want_G=True, raise_on_fail=True):
@@ -441,7 +454,8 @@ class DWFAction(torch.autograd.Function):
         S = op.norm2(chi)
         ctx.op, ctx.prec = op, prec
         ctx.save_for_backward(f, chi, U.detach())
-        return torch.tensor(S, dtype=torch.float64, device=psi.device)
+        # (a fill kernel; torch.tensor would copy S to the device and wait for it)
+        return torch.full((), S, dtype=torch.float64, device=psi.device)
 
     @staticmethod
     def backward(ctx, gS):
@@ -454,7 +468,7 @@ class DWFAction(torch.autograd.Function):
         if ctx.needs_input_grad[0]:
             grad_psi = op.unpack(op.m(chi, dag=True)) * (2.0 * g)
         if ctx.needs_input_grad[1]:
-            _, _, G = op.force(f, want_F=False, want_G=True)
+            _, G = op.force_contract(f, chi, want_F=False)
             grad_U = G * g
         return grad_psi, grad_U, None, None
 
@@ -475,7 +489,7 @@ class PseudofermionAction(torch.autograd.Function):
         f = op.pack(phi.detach(), FP64, ODD)
         S, _, G, X, _ = op.pf_force(f, tol=tol, mode=mode, want_F=False, want_G=True)
         ctx.save_for_backward(op.unpack(X, subset=ODD), G)
-        return torch.tensor(S, dtype=torch.float64, device=phi.device)
+        return torch.full((), S, dtype=torch.float64, device=phi.device)
 
     @staticmethod
     def backward(ctx, gS):
