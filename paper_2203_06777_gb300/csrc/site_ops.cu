@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, ui
       const int p0 = pad_line ? 2 * pos - 1 : 2 * pos;
       const int back = fwd ? -1 : 1;
       const int head_lane = (lane - q + (fwd ? 0 : Lsh - 1)) & 31, tail_lane = (lane - q + (fwd ? Lsh - 1 : 0)) & 31;
-      // 1 / d as an FP32 pair: the two last steps of every slice carry no error of the constant
+      // 1 / d as an FP32 pair: the last step of every slice carries no error of the constant
       const R inv_d = pws[1], inv_lo = (R)pw.inv_lo;
       const R cb = pad_head ? R(1) : pws[p0 + 1];
       R cs[STEPS > 0 ? STEPS : 1];
@@ -429,8 +429,9 @@ __global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, ui
       for (int k = 0; k < STEPS; ++k) cs[k] = pos >= (1 << k) ? pws[2 << k] : R(0);
       const R cp = head ? R(0) : inv_d;
       const R inv_dn = R(inv_den), inv_dn_lo = (R)pw.inv_den_lo;
-      auto over_den = [&](R t) { return P == P64 ? t * inv_dn : t * inv_dn + t * inv_dn_lo; };
-      auto over_d = [&](R t) { return P == P64 ? t * inv_d : t * inv_d + t * inv_lo; };
+      auto over_den = [&](R t) { return t * inv_dn + t * inv_dn_lo; };
+      // (b + y) / d without the rounding of b + y
+      auto step = [&](R b, R y) { return b * inv_d + (y * inv_d + b * inv_lo); };
 #pragma unroll
       for (int r = 0; r < RV; ++r) {
         const R a = fwd ? v[j][2 * r] : v[j][2 * r + 1];  // in line order
@@ -450,8 +451,8 @@ __global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, ui
         const R y0 = over_den(b0 - m * __shfl_sync(0xffffffffu, last, tail_lane));
         // y of the pair before, then the recurrence over the pair's own two slices
         const R prev = __shfl_sync(0xffffffffu, s1 + cb * y0, (lane + back) & 31);
-        const R ya = pad_head ? R(0) : head ? y0 : over_d(a + prev);
-        const R yb = fwd && pad_pair ? R(0) : pad_head ? y0 : over_d(b + ya);
+        const R ya = pad_head ? R(0) : head ? y0 : step(a, prev);
+        const R yb = fwd && pad_pair ? R(0) : pad_head ? y0 : step(b, ya);
         v[j][2 * r] = fwd ? ya : yb;
         v[j][2 * r + 1] = fwd ? yb : ya;
       }

@@ -1,0 +1,184 @@
+"""Every fifth-dimension extent around the limits of the kernels' dispatch, on lattices whose CTAs do not
+come out even, against the FP64 oracle: hopping term and Schur operator (even Ls to 24 and 32 are
+compiled in, the rest is generic), the fifth-dimension term (warp shuffles to 32 slice pairs, shared
+memory above and for the FP64 inverse), the force (3 to 16 pairs in registers; FP64 in block integers),
+and the integer precision conversions bit for bit.
+
+Tolerances as in test_gpu_parity: FP64 1e-12, FP32 1e-5 (force 2e-5), 16-bit storage one output
+rounding per launch (2^-11, 2^-8) with the margin used there.
+"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_06777_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+BC = (1, 1, 1, -1)
+M5, MASS = 1.8, 0.01
+TOL = {0: 1e-12, 1: 1e-5, 2: 2e-3, 3: 1.6e-2}
+TORCH = {1: torch.float32, 2: torch.float16, 3: torch.bfloat16}
+
+
+@pytest.fixture(scope="module")
+def dwf():
+    from paper_2203_06777_gb300 import dwf as mod
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    mod.load()
+    return mod
+
+
+def rel(a, b):
+    d = np.abs(a - b)
+    return float(max(np.linalg.norm(d) / np.linalg.norm(b), d.max() / np.abs(b).max()))
+
+
+def round_to(x, prec):
+    """x rounded once to the storage precision, as float64."""
+    if prec == 0:
+        return x
+    if np.iscomplexobj(x):
+        return round_to(x.real, prec) + 1j * round_to(x.imag, prec)
+    if prec == 1:
+        return x.astype(np.float32).astype(np.float64)
+    if prec == 2:
+        return x.astype(np.float16).astype(np.float64)
+    e = np.maximum(np.frexp(x)[1] - 8, -133)
+    return np.ldexp(np.rint(np.ldexp(x, -e)), e)
+
+
+def dev(x):
+    return torch.from_numpy(np.ascontiguousarray(x)).cuda()
+
+
+@pytest.mark.parametrize("dims,Ls", [((6, 2, 2, 6), 4), ((2, 6, 2, 6), 6), ((6, 6, 2, 2), 7), ((2, 2, 6, 6), 10),
+                                     ((6, 2, 6, 2), 11), ((10, 2, 2, 2), 14), ((6, 6, 6, 2), 18), ((2, 6, 6, 2), 20),
+                                     ((6, 2, 2, 2), 22), ((2, 2, 2, 6), 24), ((2, 2, 4, 2), 26), ((2, 6, 2, 2), 32),
+                                     ((6, 10, 6, 6), 12)])
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+def test_hop_and_schur_operator(dwf, oracle_lib, dims, Ls, prec):
+    U = synth.random_gauge(dims, seed=701)
+    psi = synth.random_spinor(dims, Ls, seed=702)
+    for c12 in (False, True):
+        op = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC, compress12=c12)
+        op.set_gauge(dev(U))
+        U_r = round_to(U, prec)
+        if c12:  # the third row is rebuilt from the stored two
+            U_r[..., 2, :] = np.cross(U_r[..., 0, :], U_r[..., 1, :]).conj()
+        psi_r = round_to(psi, prec)
+        out = op.unpack(op.dhop(op.pack(dev(psi), prec, dwf.FULL), dwf.FULL)).cpu().numpy()
+        assert rel(out, oracle_lib.dhop(dims, Ls, BC, U_r, psi_r)) < TOL[prec]
+        odd = oracle_lib.parity_mask(dims)[..., None, None, None]
+        f = op.pack(dev(psi), prec, dwf.ODD)
+        for dag in (False, True):
+            got = op.unpack(op.mpc(f, dag=dag), subset=dwf.ODD).cpu().numpy()
+            if dag:
+                want = psi_r * odd  # Mpc^+ from its definition by the oracle's pieces
+                te = oracle_lib.mooee(dims, Ls, M5, MASS, oracle_lib.dhop(dims, Ls, BC, U_r, want, dag=True) * ~odd,
+                                      dag=True, inverse=True)
+                want = oracle_lib.mooee(dims, Ls, M5, MASS, want, dag=True) - 0.25 * odd * oracle_lib.dhop(
+                    dims, Ls, BC, U_r, te, dag=True)
+            else:
+                want = oracle_lib.mpc(dims, Ls, M5, MASS, BC, U_r, psi_r * odd)
+            assert rel(got * odd, want * odd) < TOL[prec] * (4 if prec > 1 else 1), (c12, dag)
+        op.close()
+
+
+@pytest.mark.parametrize("Ls", [1, 2, 3, 4, 5, 9, 16, 17, 31, 32, 33, 62, 63, 64, 65, 66, 128])
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+def test_fifth_dimension_term(dwf, oracle_lib, Ls, prec):
+    dims = (2, 2, 4, 2)
+    op = dwf.GridDWF(dims, Ls, M5, MASS)
+    psi = synth.random_spinor(dims, Ls, seed=711)
+    f = op.pack(dev(psi), prec, dwf.FULL)
+    psi_r = round_to(psi, prec)
+    for dag in (False, True):
+        for inverse in (False, True):
+            ref = oracle_lib.mooee(dims, Ls, M5, MASS, psi_r, dag=dag, inverse=inverse)
+            out = op.mooee(f, dag=dag, inverse=inverse)
+            assert rel(op.unpack(out).cpu().numpy(), ref) < TOL[prec], (dag, inverse)
+            g = f.clone()
+            assert torch.equal(op.mooee(g, dag=dag, inverse=inverse, out=g), out)  # in place
+    op.close()
+
+
+@pytest.mark.parametrize("Ls", [1, 2, 5, 6, 7, 8, 9, 13, 16, 18, 23, 31, 33])
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("c12", [False, True])
+def test_force(dwf, oracle_lib, Ls, prec, c12):
+    dims = (4, 2, 6, 2)
+    U = synth.random_gauge(dims, seed=721)
+    psi = synth.random_spinor(dims, Ls, seed=722)
+    op = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC, compress12=c12)
+    op.set_gauge(dev(U))
+    f = op.pack(dev(psi), prec, dwf.FULL)
+    U_r = round_to(U, prec)
+    if c12:
+        U_r[..., 2, :] = np.cross(U_r[..., 0, :], U_r[..., 1, :]).conj()
+    S, F, G = op.force(f)
+    S_ref, F_ref, G_ref = oracle_lib.force(dims, Ls, M5, MASS, BC, U_r, round_to(psi, prec))
+    tol = 1e-12 if prec == 0 else 2e-5
+    assert abs(S - S_ref) < tol * S_ref
+    assert rel(F.cpu().numpy(), F_ref) < tol and rel(G.cpu().numpy(), G_ref) < tol
+    F2, G2 = op.force_contract(f, op.m(f))  # the contraction alone
+    assert torch.equal(F2, F) and torch.equal(G2, G)
+    op.close()
+
+
+@pytest.mark.parametrize("log2,spread", [(0, 20), (-420, 0), (420, 0), (-150, 30)])
+def test_force_fp64_magnitudes(dwf, oracle_lib, log2, spread):
+    """Slices of very different magnitude, and fields outside the integer range (IEEE products)."""
+    dims, Ls = (4, 2, 2, 4), 6
+    U = synth.random_gauge(dims, seed=731)
+    psi = synth.random_spinor(dims, Ls, seed=732)
+    psi *= np.exp2(np.random.default_rng(733).integers(-spread, spread + 1, Ls))[:, None, None]
+    op = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC)
+    op.set_gauge(dev(U))
+    _, F, G = op.force(op.pack(dev(psi * 2.0 ** log2), 0, dwf.FULL))
+    _, F_ref, G_ref = oracle_lib.force(dims, Ls, M5, MASS, BC, U, psi)
+    s = 2.0 ** -log2  # F and G are quadratic in psi
+    assert rel(F.cpu().numpy() * s * s, F_ref) < 1e-12 and rel(G.cpu().numpy() * s * s, G_ref) < 1e-12
+    op.close()
+
+
+def values(kind, n):
+    rng = np.random.default_rng(741)
+    if kind == "bits":  # every exponent, subnormals, infinities and NaN among them
+        return rng.integers(-(2 ** 63), 2 ** 63, n, dtype=np.int64).view(np.float64)
+    x = rng.normal(size=n)
+    if kind == "ties":  # halfway between neighbouring FP32 values, and just off
+        x = x.astype(np.float32).astype(np.float64) * (1 + 2.0 ** -24)
+        x[::2] = np.nextafter(x[::2], np.inf)
+        return x
+    x *= np.exp(12 * rng.normal(size=n))
+    x[:8] = [0.0, -0.0, np.inf, np.nan, 1e39, 3.4028235677973366e38, 65519.99, 65520.0]
+    return x
+
+
+@pytest.mark.parametrize("kind", ["bits", "wide", "ties"])
+@pytest.mark.parametrize("scale", [1.0, 0.75, -3.3e-5, 1e-310, 7.1e30, 0.0])
+def test_conversions_round_once(dwf, kind, scale):
+    dims, Ls = (4, 4, 4, 2), 7
+    op = dwf.GridDWF(dims, Ls, M5, MASS)
+    rv = {0: 1, 1: 2, 2: 4, 3: 4}
+
+    def by_real(t, prec):  # flat layout -> one order of the values for every precision
+        return t.reshape(-1, 24 // rv[prec], 4, (Ls + 1) // 2, rv[prec], 2).permute(0, 2, 3, 5, 1, 4).reshape(-1)
+
+    f = dev(values(kind, 2 * op.half_reals))
+    with np.errstate(all="ignore"):
+        exact = by_real(f, 0).cpu().numpy() * scale
+        for prec in (1, 2):
+            out = by_real(op.convert(f, prec, scale=scale), prec).cpu().numpy()
+            assert np.array_equal(out, exact.astype(out.dtype), equal_nan=True), prec
+        out = by_real(op.convert(f, 3, scale=scale).double(), 3).cpu().numpy()
+        finite = np.abs(exact) < 3.38e38  # (the reference below knows no overflow)
+        assert np.array_equal(out[finite], round_to(exact[finite], 3))
+        for prec in (1, 2, 3):
+            low = f.to(TORCH[prec])
+            out = by_real(op.convert(low, 0, scale=scale), 0).cpu().numpy()
+            assert np.array_equal(out, by_real(low, prec).double().cpu().numpy() * scale, equal_nan=True), prec
+    op.close()
