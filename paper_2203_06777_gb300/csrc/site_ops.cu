@@ -106,8 +106,13 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* partials, int 
 
 // ---------------------------------------------------------------- pack / unpack
 
+// One thread per 16-byte vector of the field, reading or writing the canonical values in pairs where a
+// vector holds neighbouring reals; inv_lsh = ceil(2^64 / Lsh). Pack and unpack at 16^4: FP32, Ls = 16
+// 118 -> 108 us; FP16, Ls = 16 162 -> 108 us; FP64, Ls = 12 139 -> 119 us (three 64-bit divisions per
+// vector before). Conversions in integers (as in k_convert) measured 3-14% slower here.
 template <int P>
-__global__ void k_pack_spinor(Geom g, double* canon, char* field, int parity0, int nparity, bool unpack) {
+__global__ void k_pack_spinor(Geom g, double* canon, char* field, int parity0, int nparity, bool unpack,
+                              uint64_t inv_lsh) {
   using R = RT<P>;
   constexpr int VEC = Store<P>::VEC, RV = Store<P>::RV, NCH = Store<P>::NCH;
   const long tid = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -115,34 +120,49 @@ __global__ void k_pack_spinor(Geom g, double* canon, char* field, int parity0, i
   const int Lsh = ls_half(Ls);
   const long total = (long)nparity * g.N4h * NCH * Lsh;
   if (tid >= total) return;
-  const long rem = tid / Lsh;
+  const long rem = Lsh > 1 ? (long)__umul64hi((uint64_t)tid, inv_lsh) : tid;
   const int q = (int)(tid - rem * Lsh);
   const long sitep = rem / NCH;
   const int k = (int)(rem - sitep * NCH);
-  const int ph = (int)(sitep / g.N4h);
-  const int i = (int)(sitep - (long)ph * g.N4h);
+  const int ph = sitep >= g.N4h;
+  const int i = (int)(sitep - (ph ? g.N4h : 0));
   int c[4];
   cb_coords(g, i, parity0 + ph, c);
   const long lex = c[0] + (long)g.L[0] * (c[1] + (long)g.L[1] * (c[2] + (long)g.L[2] * c[3]));
   char* fp = field + site_offset(sitep, Lsh, (size_t)Lsh * 2 * 24 * sizeof(typename Store<P>::T)) + k * chunk_stride(Lsh) +
              (size_t)q * 16;
   // value 2j + l of the vector is real RV*k + j of slice 2q + l
+  double* cp = canon + (lex * Ls + 2 * q) * 24 + RV * k;
+  const bool both = 2 * q + 1 < Ls;  // the second slice is not the pad
   if (!unpack) {
     double v[VEC];
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-      const int s = 2 * q + (e & 1);
-      v[e] = s < Ls ? canon[(lex * Ls + s) * 24 + RV * k + (e >> 1)] : 0.0;
-    }
+    for (int l = 0; l < 2; ++l)
+#pragma unroll
+      for (int j = 0; j < RV; j += RV > 1 ? 2 : 1) {
+        if constexpr (RV > 1) {
+          double2 d = make_double2(0.0, 0.0);
+          if (l == 0 || both) d = *reinterpret_cast<const double2*>(cp + l * 24 + j);
+          v[2 * j + l] = d.x;
+          v[2 * j + 2 + l] = d.y;
+        } else {
+          v[2 * j + l] = l == 0 || both ? cp[l * 24 + j] : 0.0;
+        }
+      }
     st16d<P>(fp, v);
   } else {
     R v[VEC];
     ld16<P>(fp, v);
 #pragma unroll
-    for (int e = 0; e < VEC; ++e) {
-      const int s = 2 * q + (e & 1);
-      if (s < Ls) canon[(lex * Ls + s) * 24 + RV * k + (e >> 1)] = (double)v[e];
-    }
+    for (int l = 0; l < 2; ++l)
+#pragma unroll
+      for (int j = 0; j < RV; j += RV > 1 ? 2 : 1) {
+        if (l == 1 && !both) continue;
+        if constexpr (RV > 1)
+          *reinterpret_cast<double2*>(cp + l * 24 + j) = make_double2((double)v[2 * j + l], (double)v[2 * j + 2 + l]);
+        else
+          cp[l * 24 + j] = (double)v[2 * j + l];
+      }
   }
 }
 
@@ -152,13 +172,14 @@ cudaError_t launch_pack_spinor(int prec, const Geom& g, const double* canon, voi
   const int nparity = subset == 2 ? 2 : 1;
   const long total = (long)nparity * g.N4h * (24 / (prec_vec(prec) / 2)) * ls_half(g.Ls);
   const int blocks = grid_for(total, 256);
+  const uint64_t inv = ~0ull / ls_half(g.Ls) + 1;
   double* c = const_cast<double*>(canon);
   char* f = static_cast<char*>(field);
   switch (prec) {
-    case P64: k_pack_spinor<P64><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack); break;
-    case P32: k_pack_spinor<P32><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack); break;
-    case P16: k_pack_spinor<P16><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack); break;
-    default: k_pack_spinor<PB16><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack); break;
+    case P64: k_pack_spinor<P64><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack, inv); break;
+    case P32: k_pack_spinor<P32><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack, inv); break;
+    case P16: k_pack_spinor<P16><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack, inv); break;
+    default: k_pack_spinor<PB16><<<blocks, 256, 0, st>>>(g, c, f, parity0, nparity, unpack, inv); break;
   }
   return cudaGetLastError();
 }
