@@ -1,11 +1,12 @@
 // The FP64 hopping stencil in float-float arithmetic: FP64 fields and links in memory, every
 // real carried in registers as an unevaluated sum hi + lo of two FP32 numbers.
 //
-// Why. On this part the FP64 pipe retires about two fused multiply-adds per SM and clock,
-// against 128 FP32 ones, so the FP64 kernel of dhop_kernel.cuh is bound by that pipe: it needs
-// about 20 times longer for its arithmetic than HBM needs for its bytes. A float-float operation
-// costs between 2 and 12 FP32 instructions, so the same operator in float-float runs on the wide
-// FP32 pipe instead. The format is Dekker's double-length arithmetic ("A floating-point technique
+// Why. On this part the FP64 pipe retires about two fused multiply-adds per SM and clock, against
+// 128 FP32 ones: in FP64 instructions the hop needs about 20 times longer for its arithmetic than
+// HBM needs for its bytes. A float-float operation costs between 2 and 12 FP32 instructions, so the
+// operator runs on the wide FP32 pipe instead: 261 us per 16^4 x 16 half lattice, 762 us in FP64
+// instructions. The default FP64 kernel (dhop_p64.cu) leaves the FP64 pipe too, for 64-bit integers:
+// 233 us at full FP64 precision, so the plain hop no longer gains from this one. The format is Dekker's double-length arithmetic ("A floating-point technique
 // for extending the available precision", Numer. Math. 18, 1971): a sum is formed with Knuth's
 // error-free TwoSum, a product with the FMA-based TwoProduct (the rounding error of a*b is
 // fma(a, b, -a*b) exactly). A value carries about 47 significant bits (2^-47 ~ 7e-15 relative),
@@ -14,7 +15,7 @@
 // and above 2^128 become infinite.
 //
 // Same operator, layout, thread mapping (one thread per (site, slice)), link staging and fused
-// epilogues (out = post(alpha Dhop in + beta pre(aux))) as the FP64 kernel; see there.
+// epilogues (out = post(alpha Dhop in + beta pre(aux))) as the kernels of dhop_kernel.cuh; see there.
 #include "dhop_ff.cuh"
 #include "ff_arith.cuh"
 

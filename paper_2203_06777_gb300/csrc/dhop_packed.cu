@@ -16,45 +16,43 @@ static cudaError_t launch_one(const DhopArgs& a, int threads, int blocks, size_t
       configured = smem;
     }
   }
-  {
-    // full CTAs only (the packed kernel has no tail handling); a ragged end gets one more CTA (per
-    // half) flush with the end of the lattice, launched after the first so no two writes overlap
-    // in time. a.in2 != nullptr: both halves of a full-lattice hop in the same launches.
-    // CG epilogues: partial sums [0, halves * full) from the full CTAs (CTA order), then one per
-    // half from the end CTAs, which add only the sites the full CTAs did not cover.
-    const int nsites = a.region_sites > 0 ? a.region_sites : a.g.N4h;
-    const int full = nsites / a.sites_per_cta;
-    const int halves = a.in2 ? 2 : 1;
-    DhopArgs m = a;
-    m.blocks1 = full;
-    m.red_base = 0;
-    m.own_from = 0;
-    if (full > 0) {
-      if (a.pdl) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(halves * full);
-        cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m);
-        if (e != cudaSuccess) return e;
-      } else {
-        kern<<<halves * full, threads, smem, stream>>>(m);
-      }
+  // full CTAs only (the packed kernel has no tail handling); a ragged end gets one more CTA (per
+  // half) flush with the end of the lattice, launched after the first so no two writes overlap
+  // in time. a.in2 != nullptr: both halves of a full-lattice hop in the same launches.
+  // CG epilogues: partial sums [0, halves * full) from the full CTAs (CTA order), then one per
+  // half from the end CTAs, which add only the sites the full CTAs did not cover.
+  const int nsites = a.region_sites > 0 ? a.region_sites : a.g.N4h;
+  const int full = nsites / a.sites_per_cta;
+  const int halves = a.in2 ? 2 : 1;
+  DhopArgs m = a;
+  m.blocks1 = full;
+  m.red_base = 0;
+  m.own_from = 0;
+  if (full > 0) {
+    if (a.pdl) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(halves * full);
+      cfg.blockDim = dim3(threads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = stream;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      cudaError_t e = cudaLaunchKernelEx(&cfg, kern, m);
+      if (e != cudaSuccess) return e;
+    } else {
+      kern<<<halves * full, threads, smem, stream>>>(m);
     }
-    if (a.region_sites == 0 && full * a.sites_per_cta != a.g.N4h) {
-      DhopArgs t = a;
-      t.site_base = a.g.N4h - a.sites_per_cta;
-      t.blocks1 = 1;
-      t.red_base = halves * full;
-      t.own_from = full * a.sites_per_cta;
-      kern<<<halves, threads, smem, stream>>>(t);
-    }
+  }
+  if (a.region_sites == 0 && full * a.sites_per_cta != a.g.N4h) {
+    DhopArgs t = a;
+    t.site_base = a.g.N4h - a.sites_per_cta;
+    t.blocks1 = 1;
+    t.red_base = halves * full;
+    t.own_from = full * a.sites_per_cta;
+    kern<<<halves, threads, smem, stream>>>(t);
   }
   return cudaGetLastError();
 }
