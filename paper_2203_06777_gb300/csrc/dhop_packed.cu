@@ -73,7 +73,8 @@ cudaError_t launch_dhop_pairs<DWF_PREC, DWF_PAIRS>(const DhopArgs& a, bool dag, 
     }
     return cudaErrorInvalidValue;
   }
-  if (a.pre == (dag ? PRE_MOOEE : PRE_MOOEE_DAG)) return cudaErrorInvalidValue;
+  if (a.pre == (dag ? PRE_MOOEE : PRE_MOOEE_DAG) || a.post == (dag ? POST_INV : POST_INV_DAG))
+    return cudaErrorInvalidValue;
   if (a.red && !c12 && a.pre != PRE_NONE && a.post == POST_NONE) {
     if (a.r && dag) return launch_one<true, false, EPI_PRE | EPI_AXPY>(a, threads, blocks, smem, stream);
     if (!a.r && !dag) return launch_one<false, false, EPI_PRE | EPI_NORM>(a, threads, blocks, smem, stream);
