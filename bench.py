@@ -235,11 +235,11 @@ def make_sets(dwf, torch, spec, prec, nsets, seed0, fp64_arith=0, compress12=Fal
 
 
 def launches_per_step(op, prec, dwf) -> int:
-    """Kernel launches of one full-lattice Dhop: the packed precisions run both halves in one
-    launch (plus one for the ragged end where neither the full CTAs nor a cheaper divisor divides the
-    half lattice); FP64 one launch per half."""
+    """Kernel launches of one full-lattice Dhop: one for both halves (the packed precisions one more for
+    the ragged end where neither the full CTAs nor a cheaper divisor divides the half lattice); FP64 in
+    float-float arithmetic one per half."""
     if prec == dwf.FP64:
-        return 2
+        return 2 if op.fp64_arith == dwf.FP64_ARITH_FLOAT_FLOAT else 1
     lsh = (op.Ls + 1) // 2
     spc = 128 // lsh
     if lsh == 8:
