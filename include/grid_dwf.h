@@ -263,8 +263,8 @@ int grid_dwf_face_links(grid_dwf_t* h, int precision, int out_parity, void* link
 int grid_dwf_dhop_region(grid_dwf_t* h, int precision, const void* in, void* out, int out_parity, int dag,
                          int region, const void* recv_fwd, const void* recv_bwd, const void* links_bwd);
 
-/* Measured arithmetic ceiling of the current device, the denominator of the roofline of a kernel
- * bound by its arithmetic pipe rather than by memory (the IEEE FP64 hopping term on this GPU):
+/* Measured arithmetic ceilings of the current device, to set beside the rate of a kernel that is
+ * bound by its arithmetic rather than by memory (the FP64 hopping term on this GPU):
  * FP64 FMA, scalar FP32 FMA or packed FP32x2 FMA throughput, in GFLOP/s (2 flops per FMA, 4 per
  * packed FMA) over all SMs, the best of three timed throughput loops (independent FMA chains,
  * 8 CTAs of 256 threads per SM) after one warm-up, on `stream` (NULL = legacy default stream).

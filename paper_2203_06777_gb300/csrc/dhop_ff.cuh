@@ -1,6 +1,5 @@
-// The FP64 hopping term in float-float arithmetic (dhop_ff.cu): the same DhopArgs and launch
-// shape as the FP64 kernel of dhop_kernel.cuh (one thread per (site, slice)), its own
-// shared-memory size.
+// The FP64 hopping term in float-float arithmetic (dhop_ff.cu): the DhopArgs of dhop_kernel.cuh, one
+// thread per (site, slice), its own shared-memory size.
 #pragma once
 
 #include "dhop_kernel.cuh"
