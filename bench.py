@@ -54,8 +54,8 @@ def peaks():
 
 def pipe_peaks(dwf):
     """FMA throughput of this GPU measured by the library's own loop kernels (grid_dwf_pipe_peak):
-    the FP64 ceiling is the roofline of the IEEE FP64 hopping term, which this part's FP64 pipe
-    bounds (no FP64 tensor path is used); FP32 scalar / packed FP32x2 for context."""
+    the FP64 ceiling would bound the hopping term in FP64 instructions (its products run on the integer
+    pipes instead; no FP64 tensor path is used); FP32 scalar / packed FP32x2 for context."""
     names = (("fp64_fma_gflops", dwf.PEAK_FP64_FMA), ("fp32_fma_gflops", dwf.PEAK_FP32_FMA),
              ("fp32x2_fma_gflops", dwf.PEAK_FP32X2_FMA))
     out = {k: round(dwf.pipe_peak(v), 1) for k, v in names}
@@ -520,7 +520,7 @@ def run_sweep32(dwf, torch, steps=20, warmup=3, fp64_peak=None):
 
 def run_cg32(dwf, torch):
     """Mixed-precision vs FP64 CG at 32^4 x 16, m = 0.005, exp(0.5 i H) links, one Gaussian source,
-    to a 1e-10 true residual (on by default; --no-cg32 skips it: the IEEE FP64 solve takes about 14 s)."""
+    to a 1e-10 true residual (on by default; --no-cg32 skips it: the FP64 solve takes about 5 s)."""
     spec = synth.WORKLOADS["dwf_32x32x32x32_ls16_exp0.5"]
     dims, Ls = spec["dims"], spec["Ls"]
     dev = torch.device("cuda")
@@ -848,7 +848,7 @@ def main(argv=None):
     ap.add_argument("--no-cg", action="store_true", help="skip the CG time-to-solution comparison")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
     ap.add_argument("--no-sweep", action="store_true", help="skip the 32^4 x 16 Dhop roofline sweep")
-    ap.add_argument("--no-cg32", action="store_true", help="skip the 32^4 x 16 mixed vs FP64 CG (about 25 s)")
+    ap.add_argument("--no-cg32", action="store_true", help="skip the 32^4 x 16 mixed vs FP64 CG (about 15 s)")
     ap.add_argument("--no-clock-soak", action="store_true",
                     help="skip the untimed 0.3 s run of the step before the FP32 timing (a fixed launch count, for ncu)")
     ap.add_argument("--no-force", action="store_true", help="skip the action/force and pseudofermion force timing")
