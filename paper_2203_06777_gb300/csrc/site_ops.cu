@@ -233,19 +233,20 @@ cudaError_t launch_pack_gauge(int prec, bool c12, const Geom& g, const double* c
 
 // Conversions between FP64 and the lower precisions would run on the FP64 pipe (2 lanes per SM and
 // clock; a conversion and a product by the scale take 1 clock per value against 0.5 of HBM time), so
-// the common range is done in integers, with the same single rounding:
+// the common range is done in integers, with a single rounding:
 //   down: the product of the two 53-bit significands to 62 bits, its upper word with the rest as a sticky
 //   bit, rounded to FP32 by the integer conversion (for 16-bit storage first to odd at 24 bits, so that
 //   the second rounding is exact); up: the bits rearranged.
-// Values whose result is not a normal FP32 number (zeros, infinities and NaN among them) take the FP64
-// instructions. 24^4 x 12 half field, FP64 -> FP32 with a scale: 178 -> 80 us
-// (7.1 TB/s with part of the writes still in L2; the FP64 pipe 88% busy before, idle now).
+// Values whose result is not a normal FP32 number (zeros, infinities and NaN among them), and every value
+// where the scale lies outside 2^-898 .. 2^897, take the FP64 instructions (product, then conversion).
+// 24^4 x 12 half field, FP64 -> FP32 with a scale: 178 -> 80 us (573 MB; part of the writes stays in L2;
+// the FP64 pipe 88% busy before, idle now).
 struct Scale64 {
   double v;
   uint32_t hi, lo;  // significand, left-justified
   int e;            // exponent
   uint32_t sign;
-  bool normal;
+  bool in_range;    // -898 <= e <= 896
 };
 
 __device__ __forceinline__ Scale64 make_scale64(double v) {
@@ -256,7 +257,9 @@ __device__ __forceinline__ Scale64 make_scale64(double v) {
   s.lo = l << 11;
   s.e = (int)((h >> 20) & 0x7ffu) - 1023;
   s.sign = h & 0x80000000u;
-  s.normal = s.e > -1023 && s.e < 1024;
+  // then a value whose exponent field is 0 (zero, subnormal: e - 1023) or 0x7ff (infinity, NaN: e + 1024)
+  // lies outside narrow64's range of the result's exponent, -126 .. 125
+  s.in_range = s.e >= -898 && s.e <= 896;
   return s;
 }
 
@@ -276,7 +279,7 @@ __device__ __forceinline__ typename Store<P>::T narrow64(double a, const Scale64
   const uint32_t h = (uint32_t)__double2hiint(a), l = (uint32_t)__double2loint(a);
   const uint32_t ah = __funnelshift_l(l, h, 11) | 0x80000000u, al = l << 11;
   const int k = (int)((h >> 20) & 0x7ffu) - 1023 + s.e - 30;  // value = q 2^k, q in [2^30, 2^32)
-  if ((unsigned)(k + 156) <= 251u && s.normal) {
+  if ((unsigned)(k + 156) <= 251u && s.in_range) {
     const uint64_t p = (uint64_t)ah * s.hi + __umulhi(ah, s.lo) + __umulhi(al, s.hi);
     uint32_t q = (uint32_t)(p >> 32) | ((uint32_t)p != 0);
     if constexpr (P != P32) q = (q & 0xffffff00u) | ((q & 0xffu) ? 0x100u : 0u);

@@ -182,3 +182,33 @@ def test_conversions_round_once(dwf, kind, scale):
             out = by_real(op.convert(low, 0, scale=scale), 0).cpu().numpy()
             assert np.array_equal(out, by_real(low, prec).double().cpu().numpy() * scale, equal_nan=True), prec
     op.close()
+
+
+@pytest.mark.parametrize("scale", [1e300, -1e280, 2.0 ** 897, 2.0 ** 896, 1e-290, -1e-300, 2.0 ** -899, 2.0 ** -898])
+def test_conversions_at_extreme_scales(dwf, scale):
+    """Zeros, subnormals, infinities and NaN times a scale whose exponent alone would bring them into the
+    range of normal FP32 numbers; and normal values that the scale brings there."""
+    dims, Ls = (4, 2, 2, 2), 3
+    op = dwf.GridDWF(dims, Ls, M5, MASS)
+    n = 2 * op.half_reals
+    special = [0.0, -0.0, 5e-324, -1e-310, 2.2e-308, np.inf, -np.inf, np.nan, 1.7e308]
+    x = np.resize(np.concatenate([special, values("bits", 501), np.random.default_rng(742).normal(size=64) / scale]), n)
+    # the same values at the same places of the field for every precision: one value per (site, slice)
+    psi = np.broadcast_to(x[:op.half_reals // 12].reshape(dims[::-1] + (Ls + 1, 1, 1))[..., :Ls, :, :],
+                          op.canonical_shape()).astype(np.complex128)
+    f = op.pack(dev(psi), 0, dwf.FULL)
+    with np.errstate(all="ignore"):
+        exact = x[:op.half_reals // 12].reshape(dims[::-1] + (Ls + 1,))[..., :Ls] * scale
+        for prec in (1, 2, 3):
+            low = op.convert(f, prec, scale=scale)
+            out = op.unpack(low).cpu().numpy().real
+            want = exact.astype(np.float32 if prec == 1 else np.float16) if prec < 3 else exact
+            if prec == 3:
+                finite = np.abs(exact) < 3.38e38
+                assert np.array_equal(out[finite][:, 0, 0], round_to(exact[finite], 3))
+                assert np.array_equal(np.isnan(out[..., 0, 0]), np.isnan(exact))
+            else:
+                assert np.array_equal(out[..., 0, 0], want.astype(np.float64), equal_nan=True), prec
+            rv = {1: 2, 2: 4, 3: 4}[prec]
+            assert not low.reshape(-1, 24 // rv, 4, (Ls + 1) // 2, rv, 2)[:, :, :, -1, :, 1].any()  # the pad slice
+    op.close()
