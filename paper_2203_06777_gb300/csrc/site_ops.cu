@@ -450,12 +450,12 @@ __global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, ui
       const R cb = pad_head ? R(1) : pws[p0 + 1];
       R cs[STEPS > 0 ? STEPS : 1];
 #pragma unroll
-      for (int k = 0; k < STEPS; ++k) cs[k] = pos >= (1 << k) ? pws[2 << k] : R(0);
-      const R cp = head ? R(0) : inv_d;
+      for (int k = 0; k < STEPS; ++k) cs[k] = pws[2 << k];
       const R inv_dn = R(inv_den), inv_dn_lo = (R)pw.inv_den_lo;
-      auto over_den = [&](R t) { return t * inv_dn + t * inv_dn_lo; };
-      // (b + y) / d without the rounding of b + y
-      auto step = [&](R b, R y) { return b * inv_d + (y * inv_d + b * inv_lo); };
+      auto over_den = [&](R t) { return fma(t, inv_dn, t * inv_dn_lo); };
+      // (b + y) / d without the rounding of b + y (FMAs spelled out here and below: other contractions
+      // of the same terms have up to 30% larger errors)
+      auto step = [&](R b, R y) { return fma(b, inv_d, fma(y, inv_d, b * inv_lo)); };
 #pragma unroll
       for (int r = 0; r < RV; ++r) {
         const R a = fwd ? v[j][2 * r] : v[j][2 * r + 1];  // in line order
@@ -463,18 +463,24 @@ __global__ void __launch_bounds__(256) k_mooee_vec(const char* in, char* out, ui
         const R b0 = __shfl_sync(0xffffffffu, pad_line ? b : a, head_lane);  // the line's first slice
         // S of the pair's slices: within the pair, then a scan over the pairs before it
         const R s0l = head ? R(0) : a * inv_d;
-        R s1 = pad_head ? R(0) : (b + s0l) * inv_d;
+        R s1 = pad_head ? R(0) : (head ? b : fma(a, inv_d, b)) * inv_d;
 #pragma unroll
-        for (int k = 0; k < STEPS; ++k) s1 += cs[k] * __shfl_sync(0xffffffffu, s1, (lane + back * (1 << k)) & 31);
+        for (int k = 0; k < STEPS; ++k) {
+          // beyond the line's head the shuffle reads another line: selected away, not scaled by 0 (0 x inf)
+          const R t = __shfl_sync(0xffffffffu, s1, (lane + back * (1 << k)) & 31);
+          const R f = fma(cs[k], t, s1);
+          s1 = pos >= (1 << k) ? f : s1;
+        }
         // S_{Ls-1}: on the line's last pair, its second slice unless that is the pad
         R last = s1;
         if (ODD) {
-          const R s0 = s0l + cp * __shfl_sync(0xffffffffu, s1, (lane + back) & 31);
+          const R t = __shfl_sync(0xffffffffu, s1, (lane + back) & 31);
+          const R f = fma(inv_d, t, s0l), s0 = head ? s0l : f;
           if (fwd) last = s0;
         }
-        const R y0 = over_den(b0 - m * __shfl_sync(0xffffffffu, last, tail_lane));
+        const R y0 = over_den(fma(-m, __shfl_sync(0xffffffffu, last, tail_lane), b0));
         // y of the pair before, then the recurrence over the pair's own two slices
-        const R prev = __shfl_sync(0xffffffffu, s1 + cb * y0, (lane + back) & 31);
+        const R prev = __shfl_sync(0xffffffffu, fma(cb, y0, s1), (lane + back) & 31);
         const R ya = pad_head ? R(0) : head ? y0 : step(a, prev);
         const R yb = fwd && pad_pair ? R(0) : pad_head ? y0 : step(b, ya);
         v[j][2 * r] = fwd ? ya : yb;

@@ -212,3 +212,26 @@ def test_conversions_at_extreme_scales(dwf, scale):
             rv = {1: 2, 2: 4, 3: 4}[prec]
             assert not low.reshape(-1, 24 // rv, 4, (Ls + 1) // 2, rv, 2)[:, :, :, -1, :, 1].any()  # the pad slice
     op.close()
+
+
+@pytest.mark.parametrize("Ls", [2, 3, 8, 11, 12, 16, 24, 64])
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+def test_fifth_dimension_inverse_keeps_non_finite_values_on_their_line(dwf, Ls, prec):
+    """The inverse couples the slices of one real of one site: nothing else may see an infinity or NaN."""
+    dims = (4, 2, 6, 4)
+    psi = synth.random_spinor(dims, Ls, seed=751)
+    op = dwf.GridDWF(dims, Ls, M5, MASS)
+    rng = np.random.default_rng(752)
+    where = rng.random(dims[::-1] + (4, 3)) < 0.02  # [t, z, y, x, spin, colour]
+    bad = psi.copy()
+    for idx in np.argwhere(where):
+        s = rng.integers(Ls)
+        bad[tuple(idx[:4]) + (s,) + tuple(idx[4:])] = complex([np.inf, -np.inf, np.nan][rng.integers(3)], 0.5)
+    line = np.broadcast_to(where[:, :, :, :, None], psi.shape)  # only real parts are planted
+    for dag in (False, True):
+        clean = op.unpack(op.mooee(op.pack(dev(psi), prec, dwf.FULL), dag=dag, inverse=True)).cpu().numpy()
+        out = op.unpack(op.mooee(op.pack(dev(bad), prec, dwf.FULL), dag=dag, inverse=True)).cpu().numpy()
+        assert np.array_equal(~np.isfinite(out.real), line)
+        assert np.array_equal(out.real[~line], clean.real[~line])
+        assert np.isfinite(out.imag).all() and np.array_equal(out.imag[~line], clean.imag[~line])
+    op.close()
