@@ -11,6 +11,8 @@
 // one pass. One division by n finds a unit, as a multiplication by 2^64 / n: two 64-bit divisions
 // per unit (~100 instructions each) cost the 16-bit passes most (conversion, norm and inner product of
 // BF16 full fields at 24^4 x 12: 527 -> 489 us). Pad slices (odd Ls) are zero and stay zero.
+#include <algorithm>
+
 #include "dhop_kernel.cuh"
 #include "site_ops.cuh"
 
@@ -495,20 +497,25 @@ template <int P>
 static void launch_mooee_vec(const void* in, void* out, long nsites, int Ls, bool dag, bool inverse, double d5,
                              double mass, double inv_den, const InvPowers& pw, cudaStream_t st) {
   const int Lsh = ls_half(Ls), gpw = 32 / Lsh;  // lines' vectors per warp
-  const uint32_t groups = (uint32_t)(nsites * Store<P>::NCH);
-  const int blocks = grid_for(groups, 8 * gpw * (P == P64 ? 4 : 2));
-  const char* i = static_cast<const char*>(in);
-  char* o = static_cast<char*>(out);
   int steps = 0;
   while ((1 << steps) < Lsh) ++steps;
-#define MV(S_)                                                                                                      \
-  case S_:                                                                                                          \
-    if (Ls & 1)                                                                                                     \
-      k_mooee_vec<P, S_, true><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw); \
-    else                                                                                                            \
-      k_mooee_vec<P, S_, false><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw); \
+  // 2^26 sites at most per launch, whose vectors per pair (24 per site in FP64) a 32-bit index counts
+  constexpr long STEP = 1L << 26;
+  for (long first = 0; first < nsites; first += STEP) {
+    const uint32_t groups = (uint32_t)(std::min(STEP, nsites - first) * Store<P>::NCH);
+    const int blocks = grid_for(groups, 8 * gpw * (P == P64 ? 4 : 2));
+    const size_t at = (size_t)first * Lsh * Store<P>::NCH * 16;
+    const char* i = static_cast<const char*>(in) + at;
+    char* o = static_cast<char*>(out) + at;
+#define MV(S_)                                                                                                        \
+  case S_:                                                                                                            \
+    if (Ls & 1)                                                                                                       \
+      k_mooee_vec<P, S_, true><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw);   \
+    else                                                                                                              \
+      k_mooee_vec<P, S_, false><<<blocks, 256, 0, st>>>(i, o, groups, Ls, gpw, dag, inverse, d5, mass, inv_den, pw);  \
     break;
-  switch (steps) { MV(0) MV(1) MV(2) MV(3) MV(4) MV(5) }
+    switch (steps) { MV(0) MV(1) MV(2) MV(3) MV(4) MV(5) }
+  }
 #undef MV
 }
 

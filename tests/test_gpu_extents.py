@@ -235,3 +235,24 @@ def test_fifth_dimension_inverse_keeps_non_finite_values_on_their_line(dwf, Ls, 
         assert np.array_equal(out.real[~line], clean.real[~line])
         assert np.isfinite(out.imag).all() and np.array_equal(out.imag[~line], clean.imag[~line])
     op.close()
+
+
+def test_fifth_dimension_term_of_more_than_2_32_vectors(dwf):
+    """A field with more 16-byte vectors per slice pair than 32 bits count (77 GB, in place): every site of a
+    constant field has the value of the first."""
+    dims, Ls = (128, 128, 128, 96), 2
+    nbytes = int(np.prod(dims)) * Ls * 24 * 8
+    assert int(np.prod(dims)) * 24 > 2 ** 32
+    if torch.cuda.mem_get_info()[0] < nbytes + 2 ** 33:
+        pytest.skip("needs 86 GB of free device memory")
+    small = dwf.GridDWF((2, 2, 2, 2), Ls, M5, MASS)
+    want = small.mooee(torch.ones(2 * small.half_reals, dtype=torch.float64, device="cuda"))[:4 * Ls * 24]
+    op = dwf.GridDWF(dims, Ls, M5, MASS)
+    f = torch.ones(2 * op.half_reals, dtype=torch.float64, device="cuda")
+    op.mooee(f, out=f)
+    for part in f.view(-1, 4 * Ls * 24).split(2 ** 22):
+        assert bool((part == want).all())
+    small.close()
+    op.close()
+    del f, part
+    torch.cuda.empty_cache()
