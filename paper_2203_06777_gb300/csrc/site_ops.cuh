@@ -71,12 +71,17 @@ __device__ __forceinline__ void apply_final(const Final& f, double tot, double t
 }
 
 // Sum of one value per thread over the CTA in a fixed order (warp shuffles, then the warps in
-// order), returned to thread 0.
+// order), returned to thread 0. The last warp may be short: hopping CTAs are whole sites.
 __device__ __forceinline__ double cta_sum(double v) {
   __shared__ double wsum[32];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lanes = min(32, (int)blockDim.x - 32 * warp);
+  const unsigned mask = 0xffffffffu >> (32 - lanes);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const double t = __shfl_down_sync(mask, v, off);
+    if (lane + off < lanes) v += t;
+  }
   __syncthreads();
   if (lane == 0) wsum[warp] = v;
   __syncthreads();

@@ -13,6 +13,8 @@ import torch
 
 from paper_2203_06777_gb300 import synth
 
+from .test_gpu_guards import Guarded
+
 pytestmark = pytest.mark.gpu
 
 BC = (1, 1, 1, -1)
@@ -256,3 +258,43 @@ def test_fifth_dimension_term_of_more_than_2_32_vectors(dwf):
     op.close()
     del f, part
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("dims,Ls,spc", [((6, 2, 2, 6), 10, None), ((6, 10, 6, 6), 12, None), ((6, 10, 6, 6), 12, 7),
+                                         ((2, 6, 2, 6), 7, 5), ((6, 10, 6, 22), 6, 7)])
+def test_ragged_ends_and_short_warps(dwf, oracle_lib, monkeypatch, dims, Ls, spc):
+    """CTAs whose last warp is short (120 threads in the first two cases), and sites per CTA that do not
+    divide the half lattice, so that its end takes a launch of its own (the last case with more than
+    512 partial sums in either kind of reducing launch). Sums: 48 squares per thread in FP32, all of one
+    sign, 48 x 2^-24."""
+    U, psi = synth.random_gauge(dims, seed=761, eps=0.3), synth.random_spinor(dims, Ls, seed=762)
+    plain = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC)
+    if spc:
+        monkeypatch.setenv("GRID_DWF_SITES_PER_CTA", str(spc))
+    op = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC)
+    for o in (plain, op):
+        o.set_gauge(dev(U))
+    half = op.half_reals
+    for prec in (1, 2, 3):
+        f = op.pack(dev(psi), prec, dwf.FULL)
+        calls = {"dhop": lambda o, out: o.dhop(f, dwf.FULL, out=out), "m": lambda o, out: o.m(f, dag=True, out=out),
+                 "mpc": lambda o, out: o.mpc(f[half:].clone(), out=out),
+                 "mdagm": lambda o, out: o.mdagm(f[half:].clone(), out=out)}
+        for name, call in calls.items():
+            g = Guarded(f.numel() if name in ("dhop", "m") else half, f.dtype)
+            call(op, g.t)
+            g.check(name)
+            assert torch.equal(g.t, call(plain, None)), name
+    f = op.pack(dev(psi), 1, dwf.FULL)
+    for _ in range(3):
+        S, _, _ = op.force(f, want_F=False, want_G=False)
+        assert abs(S - op.norm2(op.m(f))) < 48 * 2.0 ** -24 * S
+    b = op.pack(dev(psi), 0, dwf.FULL)
+    _, ref = plain.cg(b, tol=1e-10, maxiter=5000, mode=dwf.CG_FP64)
+    for mode in (1, 2, 3):
+        x, st = op.cg(b, tol=1e-10, maxiter=5000, mode=mode)
+        assert st.converged and st.iterations < (1.2 if mode == 1 else 2) * ref.iterations
+        r = oracle_lib.m(dims, Ls, M5, MASS, BC, U, op.unpack(x).cpu().numpy()) - psi
+        assert np.linalg.norm(r) < 1e-8 * np.linalg.norm(psi)
+    plain.close()
+    op.close()
