@@ -258,6 +258,18 @@ int hop_sites_per_cta(const grid_dwf_t* h, int prec) {
   return launch_us * (1.0 - lanes(best) / lanes(full)) < 4.0 ? best : full;
 }
 
+// A total to scal[dst] (or finalised as kind), and to pinned host memory if host is given.
+Final final_to(const grid_dwf_t* h, int kind, int dst, double* host = nullptr) {
+  return Final{reinterpret_cast<unsigned*>(h->partials + 2 * RED_BLOCKS), h->scal, kind, dst, host};
+}
+
+// The counts of a hopping launch's sums back to 0, after one of its launches (the full CTAs, a ragged end)
+// has failed: the one that ran has counted its own CTAs, and no last one has set the counts back.
+void clear_counts(grid_dwf_t* h, const CgEpilogue& epi) {
+  cudaMemsetAsync(epi.fin.count, 0, sizeof(unsigned), h->stream);
+  cudaMemsetAsync(epi.count, 0, sizeof(unsigned) * (size_t)sum_groups(epi.total), h->stream);
+}
+
 // One half-lattice hopping application with its fused epilogue.
 int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity, bool dag, int pre, int post,
               double alpha, double beta, const void* aux, const void* in2 = nullptr, void* out2 = nullptr,
@@ -362,7 +374,10 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
     case GRID_DWF_FP16: e = launch_dhop<P16>(a, dag, h->c12, threads, blocks, smem, h->stream); break;
     default: e = launch_dhop<PB16>(a, dag, h->c12, threads, blocks, smem, h->stream); break;
   }
-  if (e != cudaSuccess) return cuda_fail(h, e, "dhop launch");
+  if (e != cudaSuccess) {
+    if (epi.red) clear_counts(h, epi);
+    return cuda_fail(h, e, "dhop launch");
+  }
   return GRID_DWF_OK;
 }
 
@@ -400,11 +415,6 @@ int mdagm_impl(grid_dwf_t* h, int prec, const void* in, void* out, void* to, voi
   return GRID_DWF_OK;
 }
 
-// A total to scal[dst] (or finalised as kind), and to pinned host memory if host is given.
-Final final_to(const grid_dwf_t* h, int kind, int dst, double* host = nullptr) {
-  return Final{reinterpret_cast<unsigned*>(h->partials + 2 * RED_BLOCKS), h->scal, kind, dst, host};
-}
-
 // Workspaces of finish_grouped_sums for n partial sums: the sums, and the groups' counts (for any n of
 // this lattice; cleared once, every launch leaves them 0).
 int sums_workspace(grid_dwf_t* h, int n, CgEpilogue& epi) {
@@ -416,7 +426,14 @@ int sums_workspace(grid_dwf_t* h, int n, CgEpilogue& epi) {
   const size_t bytes = sizeof(unsigned) * (size_t)sum_groups(2 * h->g.N4h);
   RET(ws_get(h, WS_SUM_COUNTS, bytes, &p));
   epi.count = static_cast<unsigned*>(p);
-  if (fresh) CK(cudaMemsetAsync(p, 0, bytes, h->stream), "partial sums");
+  if (fresh) {
+    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, h->stream);
+    if (e != cudaSuccess) {  // not kept uncleared
+      cudaFree(p);
+      h->ws.erase(WS_SUM_COUNTS);
+      return cuda_fail(h, e, "partial sums");
+    }
+  }
   return GRID_DWF_OK;
 }
 
@@ -530,6 +547,8 @@ int grid_dwf_create(const int dims[4], int Ls, double M5, double mass, const int
   for (int k = 0; k < grid_dwf::RING && e == cudaSuccess; ++k)
     e = cudaEventCreateWithFlags(&h->ring_ev[k], cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(h->scal, 0, sizeof(double) * S_COUNT);
+  // done before any stream of the caller's runs a reduction (a non-blocking one is not ordered after this)
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     grid_dwf_destroy(h);
     return e == cudaErrorMemoryAllocation ? GRID_DWF_ERR_OOM : GRID_DWF_ERR_CUDA;
