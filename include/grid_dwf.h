@@ -112,10 +112,13 @@ int grid_dwf_set_stream(grid_dwf_t* h, void* stream);
  * force (grid_dwf_force, grid_dwf_pf_force with precision GRID_DWF_FP64); storage stays FP64, and
  * so do the vector updates and reductions of the solvers.
  * GRID_DWF_FP64_ARITH_NATIVE (the default): double precision. The hopping sum itself is formed in
- * 64-bit integer blocks (a neighbour's 24 reals of one slice share the exponent of the largest; sums
- * exact, one rounding per hop), with errors below those of IEEE arithmetic relative to the largest
- * real of the (site, slice)'s neighbours, and in IEEE double where a magnitude lies outside
- * 2^-400 .. 2^400 (infinities, NaN and subnormals included); everything else is IEEE double.
+ * 64-bit integer blocks: a neighbour's 24 reals of one slice, and a link's 18, share the exponent of
+ * the largest (57 and 58 bits below it are kept), the product of two low digits is dropped, and one
+ * rounding per hop follows. Errors are below those of IEEE arithmetic relative to the largest real of the
+ * (site, slice)'s neighbours, and at most 2^-42 (2^-49 rms) of the sum of magnitudes of any complex
+ * component's own terms. A (site, slice) whose components are too unequal for that, or a magnitude
+ * outside 2^-400 .. 2^400 (infinities, NaN and subnormals included), is computed in IEEE double. The
+ * rest of the operators, the vector updates and the reductions are IEEE double.
  * GRID_DWF_FP64_ARITH_FLOAT_FLOAT: each
  * real carried as an unevaluated sum of two floats (Dekker's double-length arithmetic: error-free
  * TwoSum and FMA-based TwoProduct), about 46 significant bits (relative error of an operator

@@ -198,18 +198,25 @@ int finish(grid_dwf_t* h, const char* where) {
   return GRID_DWF_OK;
 }
 
+// The links in the storage format of prec.
 int ensure_gauge(grid_dwf_t* h, int prec) {
   if (!h->U_canon) return fail(h, GRID_DWF_ERR_NO_GAUGE, "no gauge field set (call grid_dwf_set_gauge)");
-  if (prec == GRID_DWF_FP64 && h->fp64_arith == GRID_DWF_FP64_ARITH_NATIVE && !h->gauge_fx[1]) {
-    for (auto& q : h->gauge_fx)
-      if (!q) CK(cudaMalloc(&q, (size_t)h->g.N4h * 4 * FX_LINK_BYTES), "gauge allocation");
-    CK(launch_pack_gauge_fx(h->c12, h->g, h->U_canon, h->gauge_fx[0], h->gauge_fx[1], h->stream), "pack gauge");
-  }
   if (h->gauge[prec][0]) return GRID_DWF_OK;
   const size_t lb = link_bytes(prec_bytes(prec), h->c12);
   const size_t bytes = (size_t)h->g.N4h * 4 * lb;
   for (int p = 0; p < 2; ++p) CK(cudaMalloc(&h->gauge[prec][p], bytes), "gauge allocation");
   CK(launch_pack_gauge(prec, h->c12, h->g, h->U_canon, h->gauge[prec][0], h->gauge[prec][1], h->stream), "pack gauge");
+  return GRID_DWF_OK;
+}
+
+// The links as the hopping kernel of prec reads them: integer blocks for the native FP64 one.
+int ensure_hop_gauge(grid_dwf_t* h, int prec) {
+  if (prec != GRID_DWF_FP64 || h->fp64_arith != GRID_DWF_FP64_ARITH_NATIVE) return ensure_gauge(h, prec);
+  if (!h->U_canon) return fail(h, GRID_DWF_ERR_NO_GAUGE, "no gauge field set (call grid_dwf_set_gauge)");
+  if (h->gauge_fx[1]) return GRID_DWF_OK;
+  for (auto& q : h->gauge_fx)
+    if (!q) CK(cudaMalloc(&q, (size_t)h->g.N4h * 4 * FX_LINK_BYTES), "gauge allocation");
+  CK(launch_pack_gauge_fx(h->c12, h->g, h->U_canon, h->gauge_fx[0], h->gauge_fx[1], h->stream), "pack gauge");
   return GRID_DWF_OK;
 }
 
@@ -275,7 +282,7 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
               double alpha, double beta, const void* aux, const void* in2 = nullptr, void* out2 = nullptr,
               const void* aux2 = nullptr, const CgEpilogue& epi = CgEpilogue(),
               const HopRegion& region = HopRegion()) {
-  RET(ensure_gauge(h, prec));
+  RET(ensure_hop_gauge(h, prec));
   DhopArgs a;
   a.halo_fwd = region.halo_fwd;
   a.halo_bwd = region.halo_bwd;
@@ -343,6 +350,7 @@ int dhop_half(grid_dwf_t* h, int prec, const void* in, void* out, int out_parity
   }
   a.Ufx_out = h->gauge_fx[out_parity];
   a.Ufx_in = h->gauge_fx[1 - out_parity];
+  a.Ucanon = h->U_canon;
   a.alpha = alpha;
   a.alpha_log2 = std::ilogb(alpha);
   a.beta = beta;

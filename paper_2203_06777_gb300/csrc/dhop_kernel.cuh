@@ -90,10 +90,11 @@ struct DhopArgs {
   // Full-lattice launches: 1 to alternate the CTAs between the two halves (CTA 2b + h: CTA b of
   // half h) instead of running all CTAs of the first half first.
   int interleave;
-  // FP64 kernel (dhop_p64.cu): the links as integer blocks, output and input parity, and log2 |alpha|
-  // (alpha is a signed power of two in every launch)
+  // FP64 kernel (dhop_p64.cu; not Uout, Uin): the links as integer blocks, output and input parity, and
+  // as uploaded (canonical layout); log2 |alpha| (alpha is a signed power of two in every launch)
   const void* Ufx_out;
   const void* Ufx_in;
+  const double* Ucanon;
   int alpha_log2;
   double alpha, beta;
   double d5;       // 5 - M5

@@ -26,9 +26,21 @@
 // rounding of the stored result alone is 1.1e-16). They are relative to the largest real of the
 // neighbour's (site, slice), not to each component by itself.
 //
-// A (site, slice) one of whose neighbours or links does not fit (largest magnitude outside 2^-400 ..
-// 2^400 and not zero, which includes infinities, NaN and subnormals) is computed with IEEE FP64
-// instructions instead.
+// A component much smaller than its block's largest real keeps fewer bits than an IEEE sum of its own
+// terms would, which matters where the large reals take no part in it (other spins or, on diagonal links,
+// other colours). So the kernel adds up |re| + |im| of U h for each colour, over the x and y hops and over
+// z and t (9 of about 640 instructions per thread and hop; Mpc^+ Mpc at 16^4 x 16 1016 -> 1050 us), and a
+// (site, slice) with a complex component for which neither sum reaches an eighth of the smallest product of
+// two blocks' largest reals (2^53 accumulator units) is computed with IEEE FP64 instructions. The errors
+// above are at most 92 units per real over the eight hops (1 unit rms), so a component's error is at most
+// 2^-42 (2^-49 rms) of the sum of its terms' magnitudes, at the limit; typically they sum to 8 x 2^53
+// units. Gaussian fields stay above the limit (none of 4e5 simulated sites below), propagators on random
+// and on smooth links nearly everywhere (3e-5 of the sites of an 8^4 x 8 point source's); a limit of 2^53
+// would send 17-43% of the latter to IEEE instructions. Components all of whose terms are 0 (a source's
+// empty spins and colours) come out exactly 0 either way and stay.
+//
+// IEEE instructions also where a neighbour or link does not fit (largest magnitude outside 2^-400 ..
+// 2^400 and not zero, which includes infinities, NaN and subnormals).
 //
 // Code shape. Two threads (neighbouring lanes) per (site, slice), one for each spin k of the half
 // spinor: thread k forms h_k, multiplies it by the link and accumulates it into spin k and into the
@@ -44,12 +56,13 @@ namespace gdwf {
 namespace {
 
 constexpr int FX_BAD = -1;                // link exponent of a link that does not fit
-constexpr int FX_HOP_BYTES = FX_LINK_BYTES;  // staged: 9 complex entries, then {exponent, neighbour}
+constexpr int FX_MIN_TERMS = 1 << 18;     // 2^50 accumulator units, an eighth of the smallest product of two blocks
+constexpr int FX_HOP_BYTES = FX_LINK_BYTES;  // staged: 9 complex entries, then {exponent, neighbour, entries not 0}
 // 16 bytes of padding per site: two sites read by one warp fall on different banks
 constexpr int FX_SITE_BYTES = 8 * FX_HOP_BYTES + 16;
 
 // Links of every site as blocks of digits: entry (a, b) is {re d1, re d0, im d1, im d0}, then the
-// exponent. One thread per link.
+// exponent and which entries are not 0. One thread per link.
 template <bool C12>
 __global__ void k_pack_gauge_fx(Geom g, const double* canon, char* Ue, char* Uo) {
   const long tid = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -73,9 +86,14 @@ __global__ void k_pack_gauge_fx(Geom g, const double* canon, char* Ue, char* Uo)
     emax = (uint32_t)FX_LO << 20;
   }
   int4* dst = reinterpret_cast<int4*>((p ? Uo : Ue) + ((size_t)i * 4 + mu) * FX_LINK_BYTES);
+  int nonzero = 0, nonzero_t = 0;  // bit 3 a + b (b + 3 a of the adjoint): entry (a, b) is not 0
 #pragma unroll
   for (int j = 0; j < 9; ++j) {
     int4 d = make_int4(0, 0, 0, 0);
+    if (!fx_all_zero<2>(u + 2 * j)) {
+      nonzero |= 1 << j;
+      nonzero_t |= 1 << (j % 3 * 3 + j / 3);
+    }
     if (e != FX_BAD) {
       const int rh = __double2hiint(u[2 * j]), ih = __double2hiint(u[2 * j + 1]);
       fx_magnitude<9>((uint32_t)rh, (uint32_t)__double2loint(u[2 * j]), emax, d.x, d.y);
@@ -85,47 +103,112 @@ __global__ void k_pack_gauge_fx(Geom g, const double* canon, char* Ue, char* Uo)
     }
     dst[j] = d;
   }
-  dst[9] = make_int4(e, 0, 0, 0);
+  dst[9] = make_int4(e, 0, nonzero, nonzero_t);
 }
 
-// The hopping sum of one (site, slice) in IEEE FP64, for inputs outside the integer range.
+// The reals of a neighbour's spins psi_k (u) and psi_{p_k} (l) that thread k projects along mu, the second
+// with real and imaginary parts exchanged where the projector multiplies it by i (x and z).
+__device__ __forceinline__ void fx_load(const char* site, int mu, int k, size_t cs, double* u, double* l) {
+  const char* ub = site + 6 * k * cs;
+  const char* lb = site + (mu < 2 ? 18 - 6 * k : 12 + 6 * k) * cs;
+  const size_t o0 = (mu & 1) == 0 ? cs : 0, o1 = cs - o0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    u[2 * c] = __ldg(reinterpret_cast<const double*>(ub + (2 * c) * cs));
+    u[2 * c + 1] = __ldg(reinterpret_cast<const double*>(ub + (2 * c + 1) * cs));
+    l[2 * c] = __ldg(reinterpret_cast<const double*>(lb + (2 * c) * cs + o0));
+    l[2 * c + 1] = __ldg(reinterpret_cast<const double*>(lb + (2 * c) * cs + o1));
+  }
+}
+
+// Signs of the projection of spin k: h_k = u + l with the real (bit 0) and imaginary (bit 1) part of l
+// subtracted; plus: projector (1 + gamma_mu), otherwise (1 - gamma_mu). As a nibble {k=0 re, k=0 im, k=1 re,
+// k=1 im} for (1 + gamma), complemented for (1 - gamma).
+__device__ __forceinline__ uint32_t fx_signs(int mu, int k, bool plus) {
+  return (((0x063Au >> (4 * mu)) & 15u) ^ (plus ? 0u : 15u)) >> (2 * k);
+}
+
+// Whether the lower spin's term, U h_k (y, t) or i U h_k (x, z), is subtracted: (1 + gamma) has x +,
+// y k=0 - k=1 +, z k=0 + k=1 -, t +.
+__device__ __forceinline__ bool fx_lower_minus(int mu, int k, bool plus) {
+  return !plus ^ (mu == 1 ? k == 0 : mu == 2 ? k == 1 : false);
+}
+
+// The hopping sum of one (site, slice) in IEEE FP64, for inputs outside the integer range or precision: lane
+// k's spin k, then its part of the lower spins from the x and y hops and from the z and t hops. The links
+// are those that the integer blocks were made of (canonical layout).
 template <bool C12>
-__device__ __noinline__ void hop_ieee(const DhopArgs& a, int out_parity, const char* in, const char* Uo, const char* Ui,
-                                      int site, int s, bool dag, double* out) {
-  constexpr int LB = link_bytes(8, C12);
+__device__ __noinline__ void hop_ieee(const DhopArgs& a, int out_parity, const char* in, int site, int k, bool dag,
+                                      double* out) {
   const int Lsh = ls_half(a.g.Ls);
-  const size_t site_bytes = (size_t)Lsh * 2 * 24 * 8;
+  const size_t site_bytes = (size_t)Lsh * 2 * 24 * 8, cs = chunk_stride(Lsh);
   int c[4];
   cb_coords(a.g, site, out_parity, c);
-  double acc[24];
+  const long stride[4] = {1, a.g.L[0], (long)a.g.L[0] * a.g.L[1], (long)a.g.L[0] * a.g.L[1] * a.g.L[2]};
+  const long lex = c[0] + c[1] * stride[1] + c[2] * stride[2] + c[3] * stride[3];
+  double acc[18];
 #pragma unroll
-  for (int r = 0; r < 24; ++r) acc[r] = 0;
+  for (int r = 0; r < 18; ++r) acc[r] = 0;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
     for (int back = 0; back < 2; ++back) {
       int ph;
       const int j = cb_neighbour(a.g, site, c, mu, back == 0, ph);
-      double u[18], psi[24], h[12], uh[12];
-      load_link<P64, C12>((back ? Ui + ((size_t)j * 4 + mu) * LB : Uo + ((size_t)site * 4 + mu) * LB), u);
-      load_lane64<0>(in + site_offset(j, Lsh, site_bytes), s, Lsh, psi);
+      const long before = c[mu] > 0 ? lex - stride[mu] : lex + (a.g.L[mu] - 1) * stride[mu];
+      const double* link = a.Ucanon + ((back ? before : lex) * 4 + mu) * 18;
+      double u[18], h[6], l[6];
+#pragma unroll
+      for (int r = 0; r < (C12 ? 12 : 18); ++r) u[r] = __ldg(link + r);
+      if (C12) reconstruct_row2(u);
+      fx_load(in + site_offset(j, Lsh, site_bytes), mu, k, cs, h, l);
+      const bool plus = (back == 0) == dag;
+      const uint32_t neg = fx_signs(mu, k, plus);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) h[r] += (neg >> (r & 1)) & 1u ? -l[r] : l[r];
       const double cph = ph < 0 ? -a.alpha : a.alpha;
-      const bool plus = (back == 0) == dag;  // projector (1 + gamma) or (1 - gamma)
-      if (plus)
-        project<+1>(mu, psi, h);
-      else
-        project<-1>(mu, psi, h);
-      if (back)
-        su3_mul<true>(u, h, uh);
-      else
-        su3_mul<false>(u, h, uh);
-      if (plus)
-        accumulate<+1>(mu, uh, cph, acc);
-      else
-        accumulate<-1>(mu, uh, cph, acc);
+      const double clow = fx_lower_minus(mu, k, plus) ? -cph : cph;
+      double* low = acc + (mu < 2 ? 6 : 12);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        double re = 0, im = 0;
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const int e = back ? b * 3 + r : r * 3 + b;
+          const double ur = u[2 * e], ui = back ? -u[2 * e + 1] : u[2 * e + 1];
+          re = fma(ur, h[2 * b], re);
+          im = fma(ur, h[2 * b + 1], im);
+          re = fma(-ui, h[2 * b + 1], re);
+          im = fma(ui, h[2 * b], im);
+        }
+        acc[2 * r] = fma(cph, re, acc[2 * r]);
+        acc[2 * r + 1] = fma(cph, im, acc[2 * r + 1]);
+        low[2 * r] = (mu & 1) == 0 ? fma(-clow, im, low[2 * r]) : fma(clow, re, low[2 * r]);
+        low[2 * r + 1] = (mu & 1) == 0 ? fma(clow, re, low[2 * r + 1]) : fma(clow, im, low[2 * r + 1]);
+      }
     }
   }
-  for (int r = 0; r < 24; ++r) out[r] = acc[r];
+  for (int r = 0; r < 18; ++r) out[r] = acc[r];
+}
+
+// Which colours of U h_k have a term that is not 0: bits 0 to 2 over the x and y hops, 3 to 5 over z and t.
+__device__ __noinline__ int fx_terms(const char* in, const unsigned char* lsm, int k, int Lsh, size_t site_bytes) {
+  int terms = 0;
+#pragma unroll 1
+  for (int hop = 0; hop < 8; ++hop) {
+    const int* staged = reinterpret_cast<const int*>(lsm + hop * FX_HOP_BYTES + 9 * 16);
+    const int nb = staged[1], entries = staged[2];
+    double u[6], l[6];
+    fx_load(in + site_offset(nb, Lsh, site_bytes), hop >> 1, k, chunk_stride(Lsh), u, l);
+    int h = 0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (!fx_all_zero<2>(u + 2 * c) || !fx_all_zero<2>(l + 2 * c)) h |= 1 << c;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if ((entries >> (3 * c)) & h) terms |= 1 << (hop < 4 ? c : c + 3);
+  }
+  return terms;
 }
 
 // v >> d for 0 <= d <= 31
@@ -182,6 +265,7 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
         int slot = e;
         if (e == 9) {
           d.y = nb;
+          if (!fwd) d.z = d.w;
         } else {
           const int sr = ph, si = fwd ? ph : -ph;
           d.x *= sr;
@@ -207,33 +291,29 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
     const char* in = in_field + (size_t)s * 8;
     // the lanes of this warp (the last warp of a CTA may be short)
     const uint32_t lanes = (int)blockDim.x - (tid & ~31) >= 32 ? 0xffffffffu : (1u << (blockDim.x & 31)) - 1u;
-    // h_k = psi_k +- (1 or i) psi_{p_k} of hop's neighbour: both spins of this lane, the second
-    // with real and imaginary parts exchanged where it is multiplied by i (x and z)
-    auto load_hop = [&](int hop, double* u, double* l) {
-      const int mu = hop >> 1;
-      const int nb = *reinterpret_cast<const int*>(lsm + hop * FX_HOP_BYTES + 9 * 16 + 4);
-      const char* blk = in + site_offset(nb, Lsh, site_bytes);
-      const char* ub = blk + 6 * k * cs;
-      const char* lb = blk + (mu < 2 ? 18 - 6 * k : 12 + 6 * k) * cs;
-      const size_t o0 = (mu & 1) == 0 ? cs : 0, o1 = cs - o0;
+    // |re| + |im| of U h_k for each colour (2^32 accumulator units), summed over the x and y hops, then over z
+    // and t; which of the former sums are large enough
+    int terms[3] = {0, 0, 0}, large_xy = 0;
+    auto large_terms = [&] {
+      int m = 0;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        u[2 * c] = __ldg(reinterpret_cast<const double*>(ub + (2 * c) * cs));
-        u[2 * c + 1] = __ldg(reinterpret_cast<const double*>(ub + (2 * c + 1) * cs));
-        l[2 * c] = __ldg(reinterpret_cast<const double*>(lb + (2 * c) * cs + o0));
-        l[2 * c + 1] = __ldg(reinterpret_cast<const double*>(lb + (2 * c) * cs + o1));
-      }
+      for (int c = 0; c < 3; ++c) m |= terms[c] >= FX_MIN_TERMS ? 1 << c : 0;
+      return m;
     };
 #pragma unroll 1
     for (int hop = 0; hop < 8; ++hop) {
       const int mu = hop >> 1;
-      // signs of the second spin's parts, as a nibble {k=0 re, k=0 im, k=1 re, k=1 im} (bit set:
-      // subtract) for the (1 + gamma) projector, complemented for (1 - gamma)
+      if (hop == 4) {
+        large_xy = large_terms();
+#pragma unroll
+        for (int c = 0; c < 3; ++c) terms[c] = 0;
+      }
       const bool plus = ((hop & 1) == 0) == dag;  // projector (1 + gamma_mu) or (1 - gamma_mu)
       const int lexp = *reinterpret_cast<const int*>(lsm + hop * FX_HOP_BYTES + 9 * 16);
-      const uint32_t neg = (((0x063Au >> (4 * mu)) & 15u) ^ (plus ? 0u : 15u)) >> (2 * k);
+      const int nb = *reinterpret_cast<const int*>(lsm + hop * FX_HOP_BYTES + 9 * 16 + 4);
+      const uint32_t neg = fx_signs(mu, k, plus);
       double u[6], l[6];
-      load_hop(hop, u, l);
+      fx_load(in + site_offset(nb, Lsh, site_bytes), mu, k, cs, u, l);
       // one block exponent for the neighbour's 24 reals (the two lanes hold 12 each)
       uint32_t emax = max(fx_max_hi<6>(u), fx_max_hi<6>(l)) & 0x7ff00000u;
       emax = max(emax, __shfl_xor_sync(lanes, emax, 1));
@@ -258,6 +338,9 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
           lxy[r] = (lxy[r] + half) >> sh;
           lzt[r] = (lzt[r] + half) >> sh;
         }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) terms[c] >>= min(sh, 31);
+        large_xy = 0;
         eacc = er + 4;
       }
       int d = eacc - er;
@@ -282,9 +365,7 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
           d0[i] = l0 * sl + u0 * su;
         }
       }
-      // sign of the lower spin's term: (1 + gamma): x +, y k=0 - k=1 +, z k=0 + k=1 -, t +
-      const bool minus = !plus ^ (mu == 1 ? k == 0 : mu == 2 ? k == 1 : false);
-      const long long sm = minus ? -1 : 0;  // 0 or -1
+      const long long sm = fx_lower_minus(mu, k, plus) ? -1 : 0;
       const int4* us = reinterpret_cast<const int4*>(lsm + hop * FX_HOP_BYTES);
       long long v[6];
 #pragma unroll
@@ -315,6 +396,8 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
       }
 #pragma unroll
       for (int r = 0; r < 6; ++r) up[r] += v[r];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) terms[c] += abs((int)(v[2 * c] >> 32)) + abs((int)(v[2 * c + 1] >> 32));
       // lower spin += +-(v_r + i v_i) (y, t) or +-i (v_r + i v_i) (x, z)
 #define FX_LOWER(acc, re, m_re, im, m_im)                        \
   for (int c = 0; c < 6; c += 2) {                               \
@@ -348,19 +431,29 @@ __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs 
       x[r] = to_double(up[r]);
       x[6 + r] = to_double(lzt[r] + __shfl_xor_sync(lanes, lxy[r], 1));  // eacc is the same in both lanes
     }
-    const int bad_other = __shfl_xor_sync(lanes, (int)bad, 1);  // by both lanes, whatever their own flag
-    if (bad || bad_other != 0) {
-      double t[24];
-      const char* Uo = static_cast<const char*>(second ? a.Uin : a.Uout);
-      const char* Ui = static_cast<const char*>(second ? a.Uout : a.Uin);
+    // components whose terms are too small for the accumulator's unit: spin k in bits 0 to 2, spin 2 + k
+    // (which has the other lane's x and y hops) in bits 3 to 5; bit 6: outside the integer range
+    const int large_zt = large_terms(), large_other = __shfl_xor_sync(lanes, large_xy, 1);
+    int flags = s < Ls ? ((large_xy | large_zt) | (large_other | large_zt) << 3) ^ 63 : 0;
+    if (bad) flags |= 64;
+    const int flags_other = __shfl_xor_sync(lanes, flags, 1);  // by both lanes, whatever their own
+    bool ieee = ((flags | flags_other) & 64) != 0;
+    const uint32_t pair = 3u << (tid & 30);
+    if (!ieee && (flags | flags_other) != 0) {  // both lanes of the pair come here
+      const int own = fx_terms(in, lsm, k, Lsh, site_bytes), other = __shfl_xor_sync(pair, own, 1);
+      const int need = flags & ((own | (own >> 3)) & 7 | ((own & 56) | (other & 7) << 3));
+      ieee = (need | __shfl_xor_sync(pair, need, 1)) != 0;
+    }
+    if (ieee) {
+      double t[18];
       if (c12)
-        hop_ieee<true>(a, out_parity, in_field, Uo, Ui, site, s, dag, t);
+        hop_ieee<true>(a, out_parity, in, site, k, dag, t);
       else
-        hop_ieee<false>(a, out_parity, in_field, Uo, Ui, site, s, dag, t);
+        hop_ieee<false>(a, out_parity, in, site, k, dag, t);
 #pragma unroll
       for (int r = 0; r < 6; ++r) {
-        x[r] = k ? t[6 + r] : t[r];
-        x[6 + r] = k ? t[18 + r] : t[12 + r];
+        x[r] = t[r];
+        x[6 + r] = t[12 + r] + __shfl_xor_sync(pair, t[6 + r], 1);
       }
     }
   }

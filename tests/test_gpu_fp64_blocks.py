@@ -102,3 +102,63 @@ def test_zero_field(dwf):
     U = synth.random_gauge(DIMS, seed=48)
     out = apply(dwf, U, np.zeros(DIMS[::-1] + (5, 4, 3), dtype=np.complex128), 5, False)
     assert np.all(out == 0)
+
+
+def hop_terms(U, psi, dag):
+    """Sum of the magnitudes of the terms of every complex component of the hop: over the eight hops of
+    a site, sum_b |U_ab| |h_b| with h the projected neighbour (its lower spins repeat the upper ones)."""
+    sign = 1 if dag else -1  # forward projector (1 + sign gamma), backward (1 - sign gamma)
+    total = np.zeros(psi.shape)
+    partner = {0: (3, 2), 1: (3, 2), 2: (2, 3), 3: (2, 3)}
+    coeff = {0: (-1j, -1j), 1: (-1, 1), 2: (-1j, 1j), 3: (1, 1)}  # h_k = psi_k + s coeff psi_partner, k = 0, 1
+    for mu in range(4):
+        axis = 3 - mu
+        for back in (0, 1):
+            nb = np.roll(psi, 1 if back else -1, axis)
+            link = U[..., mu, :, :]
+            link = np.roll(link, 1, axis).swapaxes(-1, -2) if back else link
+            s = -sign if back else sign
+            for k in (0, 1):
+                h = nb[..., k, :] + s * coeff[mu][k] * nb[..., partner[mu][k], :]
+                t = np.einsum("tzyxab,tzyxsb->tzyxsa", np.abs(link), np.abs(h))
+                total[..., k, :] += t
+                total[..., partner[mu][k], :] += t
+    return total
+
+
+def graded(kind, psi, U):
+    """Fields whose components differ in size by more than a block of integers with one exponent holds, on
+    links that leave some of the small ones apart."""
+    psi, U = psi.copy(), U.copy()
+    if kind == "colours":
+        psi *= np.exp2([0, -20, -40])
+        U[...] = np.eye(3)
+    elif kind == "spins":  # spin 1 takes no part in spin 0's hops
+        psi *= np.exp2([-30, 0, -30, -30])[:, None]
+    elif kind == "colours and zeros":
+        psi *= np.array([1, 0, 2.0 ** -70])
+        U[...] = np.eye(3)
+    elif kind == "links":
+        U[...] = np.diag(np.exp2([0, -25, -50]))
+    elif kind == "links and a little mixing":
+        U[...] = np.eye(3) + 2.0 ** -58 * U
+        psi *= np.array([1, 0, 0])
+    elif kind == "one spin":
+        psi *= np.array([0, 0, 1, 0])[:, None]
+    return psi, U
+
+
+@pytest.mark.parametrize("kind", ["equal", "colours", "spins", "colours and zeros", "links",
+                                  "links and a little mixing", "one spin"])
+@pytest.mark.parametrize("Ls", [3, 8])
+def test_small_components_beside_large_ones(dwf, oracle_lib, kind, Ls):
+    """Every complex component to a precision relative to its own terms. Oracle: at most 24 roundings of a
+    term, 24 x 2^-53. Block integers: a hop's truncations and its rounding add up to 11 units of the
+    accumulator per real, with the accumulator's own shifts 92 for eight hops, sqrt(2) x 92 for the modulus,
+    and they are used only where the |re| + |im| of the hops sum to 2^50 units or more, the moduli of the
+    terms to 2^49.5: 1450 x 2^-53. Together 1500 x 2^-53 of the sum of magnitudes."""
+    psi, U = graded(kind, synth.random_spinor(DIMS, Ls, seed=51), synth.random_gauge(DIMS, seed=52))
+    for dag in (False, True):
+        ref = oracle_lib.dhop(DIMS, Ls, BC, U, psi, dag=dag)
+        err = np.abs(apply(dwf, U, psi, Ls, dag) - ref)
+        assert np.all(err <= 1500 * 2.0 ** -53 * hop_terms(U, psi, dag))
