@@ -118,7 +118,9 @@ int grid_dwf_set_stream(grid_dwf_t* h, void* stream);
  * (site, slice)'s neighbours, and at most 2^-42 (2^-49 rms) of the sum of magnitudes of any complex
  * component's own terms. A (site, slice) whose components are too unequal for that, or a magnitude
  * outside 2^-400 .. 2^400 (infinities, NaN and subnormals included), is computed in IEEE double. The
- * rest of the operators, the vector updates and the reductions are IEEE double.
+ * FP64 force forms its outer products and their sums over the slices in the same way, and in IEEE double
+ * any entry far below the largest product of its site's slices. The rest of the operators and of the
+ * force, the vector updates and the reductions are IEEE double.
  * GRID_DWF_FP64_ARITH_FLOAT_FLOAT: each
  * real carried as an unevaluated sum of two floats (Dekker's double-length arithmetic: error-free
  * TwoSum and FMA-based TwoProduct), about 46 significant bits (relative error of an operator

@@ -405,10 +405,18 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
 // link algebra of all four directions follows at the end, in FP64, 36 entries per site (direction by
 // direction, with 36 of 128 threads at work between barriers: force call at 16^4 x 16 1612 us; with
 // FP64 products 2520 us; now 1288 us, of which M psi is 470 us). Integer instructions and the barriers
-// around the slice sums bound it now. A block of sites with a magnitude outside the integer range takes force_products_ieee
-// instead, for all its slices.
+// around the slice sums bound it now.
+// IEEE instructions instead: for a block of sites with a magnitude outside the integer range, all its
+// slices (force_products_ieee); and for an entry of B1 or B2 whose slices' |re| + |im| sum to less than an
+// eighth of the smallest product of two blocks' largest reals (force_entry_ieee), since the integers'
+// errors, relative to that product, could be large beside it (colours or spins of very different size).
+// Above that limit a real's error is at most (81 + Ls / 2) 2^(n - 53) of that sum, n = ceil(log2 Ls).
+// Gaussian fields with Ls = 1 / 2: 0.5% / 8e-6 of the entries lie below it, with 3 and more none of 1e5
+// simulated ones. Force call at 16^4, without and with the check: Ls = 16 1287 and 1311 us, Ls = 2 430 and
+// 442 us, Ls = 1 435 and 510 us.
 constexpr int FORCE_FX_STRIDE = 19;  // 64-bit values per (slice, term): 18, odd so that stores spread over the banks
 constexpr int FORCE_FX_OWN = 25;     // digit pairs per thread of the own spinor: 24, odd for the same reason
+constexpr int FORCE_FX_MIN_TERMS = 1 << 21;  // 2^53 of 2^56 units, an eighth of the smallest product
 // Threads and sites per CTA at most (Ls > 32: one site). 256 threads, two CTAs per SM instead of four,
 // wait longer at the barriers: 1382 us.
 constexpr int FORCE_FX_THREADS = 128, FORCE_FX_SITES = 16;
@@ -442,6 +450,41 @@ __device__ __noinline__ void force_products_ieee(const char* psi_x, const char* 
         }
     }
   }
+}
+
+// One real of a site's slice sums in IEEE FP64 (im: the imaginary part of entry (a, b) of B1, or with
+// term = 1 of B2), for a sum that the block integers would give fewer bits than its own products have.
+__device__ __noinline__ double force_entry_ieee(const Geom& g, const char* psi, const char* chi, int p, int i, int mu,
+                                                int term, int a, int b, int im) {
+  const int Lsh = ls_half(g.Ls);
+  const size_t site_bytes = (size_t)Lsh * 2 * 24 * 8, cs = chunk_stride(Lsh);
+  const size_t half_bytes = (size_t)g.N4h * site_bytes;
+  int c[4], ph;
+  cb_coords(g, i, p, c);
+  const size_t own = p * half_bytes + site_offset(i, Lsh, site_bytes);
+  const size_t nb = (1 - p) * half_bytes + site_offset(cb_neighbour(g, i, c, mu, true, ph), Lsh, site_bytes);
+  const char* x = psi + (term ? own : nb);
+  const char* y = chi + (term ? nb : own);
+  const uint32_t neg = ((0x063Au >> (4 * mu)) & 15u) ^ (term ? 0u : 15u);  // as in k_force_fx
+  const int swap = (mu & 1) == 0;
+  // part r (0 re, 1 im) of the projected spin h, colour col
+  auto half_spin = [&](const char* f, int h, int col, int r) {
+    const int upper = 6 * h + 2 * col + r, lower = (mu < 2 ? 18 - 6 * h : 12 + 6 * h) + 2 * col + (swap ? 1 - r : r);
+    const double u = __ldg(reinterpret_cast<const double*>(f + upper * cs));
+    const double l = __ldg(reinterpret_cast<const double*>(f + lower * cs));
+    return (neg >> (2 * h + r)) & 1u ? u - l : u + l;
+  };
+  double sum = 0;
+  for (int s = 0; s < g.Ls; ++s, x += 8, y += 8) {
+    double v = 0;
+    for (int h = 0; h < 2; ++h) {
+      const double xr = half_spin(x, h, a, 0), xi = half_spin(x, h, a, 1);
+      const double yr = half_spin(y, h, b, 0), yi = half_spin(y, h, b, 1);
+      v = im ? fma(xi, yr, fma(-xr, yi, v)) : fma(xr, yr, fma(xi, yi, v));
+    }
+    sum += v;
+  }
+  return sum;
 }
 
 inline size_t force_fx_smem(int nsg, int spc) {
@@ -622,11 +665,22 @@ __global__ void __maxnreg__(128) k_force_fx(const Geom g, const char* psi, const
         const int kk = term ? (b * 3 + a) * 2 + (k & 1) : k;
         const long long* src = part + ((size_t)sl * nsg + term) * FORCE_FX_STRIDE + kk;
         long long tot = 0;
-        for (int q = 0; q < Lsp; ++q) tot += src[q * (2 * FORCE_FX_STRIDE)];
+        int terms = 0;  // sum of the slices' magnitudes (2^32 of their units)
+        for (int q = 0; q < Lsp; ++q) {
+          const long long c = src[q * (2 * FORCE_FX_STRIDE)];
+          tot += c;
+          terms += abs((int)(c >> 32));
+        }
         v = (double)tot;
         const int ex = e_sm[2 * sl + term] + sum_shift - 2102;
         if (tot != 0) v = __hiloint2double(__double2hiint(v) + (ex << 20), __double2loint(v));
         if (term && (k & 1)) v = -v;
+        if (terms < (FORCE_FX_MIN_TERMS >> sum_shift)) {  // then the other part of the complex number counts, too
+          const int other = (kk ^ 1) - kk;
+          for (int q = 0; q < Lsp; ++q) terms += abs((int)(src[q * (2 * FORCE_FX_STRIDE) + other] >> 32));
+        }
+        if (terms < (FORCE_FX_MIN_TERMS >> sum_shift))
+          v = force_entry_ieee(g, psi, chi, p, first + sl, mu, term, a, b, k & 1);
       } else {
         const double* src = reinterpret_cast<const double*>(part + (size_t)sl * nsg * FORCE_FX_STRIDE) + e;
         for (int q = 0; q < Lsp; ++q) v += src[q * (2 * FORCE_FX_STRIDE)];

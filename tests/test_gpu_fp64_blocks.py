@@ -162,3 +162,19 @@ def test_small_components_beside_large_ones(dwf, oracle_lib, kind, Ls):
         ref = oracle_lib.dhop(DIMS, Ls, BC, U, psi, dag=dag)
         err = np.abs(apply(dwf, U, psi, Ls, dag) - ref)
         assert np.all(err <= 1500 * 2.0 ** -53 * hop_terms(U, psi, dag))
+
+
+@pytest.mark.parametrize("Ls", [1, 2, 6, 16])
+def test_force_of_small_colours_beside_large_ones(dwf, oracle_lib, Ls):
+    """Unit links keep the colours apart: entry (a, b) of the gradient is a sum of products of psi's and
+    chi's colours a and b, of any size beside the others. 1e-12 as for whole FP64 fields elsewhere."""
+    size = np.exp2([0, -20, -40])
+    U = synth.unit_gauge(DIMS)
+    psi = synth.random_spinor(DIMS, Ls, seed=53) * size
+    op = dwf.GridDWF(DIMS, Ls, M5, MASS, bc=BC)
+    op.set_gauge(torch.from_numpy(U).cuda())
+    _, _, G = op.force(op.pack(torch.from_numpy(psi).cuda(), 0, dwf.FULL))
+    _, _, ref = oracle_lib.force(DIMS, Ls, M5, MASS, BC, U, psi)
+    s = size[:, None] * size
+    assert np.all(np.abs(G.cpu().numpy() - ref) / s <= 1e-12 * np.abs(ref / s).max())
+    op.close()
