@@ -25,6 +25,7 @@
 // the FP32 fields and block sums anyway. FP64 fields: k_force_fx below. F and G are written
 // in the canonical FP64 layout [t][z][y][x][mu][3][3].
 #include <algorithm>
+#include <cstdint>
 
 #include "dhop_kernel.cuh"
 #include "ff_arith.cuh"
@@ -891,7 +892,9 @@ cudaError_t launch_force(int prec, bool c12, const Geom& g, const void* psi, con
     kern<<<gr, n2 * s2, sm, st>>>(g, ps, ch, e, o, F, G, coef, n2, s2, shift);
     return cudaGetLastError();
   }
-  if (prec == P32 && Lsh >= 3 && Lsh <= 16) {
+  // (k_force_reg stores F and G in pairs of reals)
+  const bool aligned = (reinterpret_cast<uintptr_t>(F) | reinterpret_cast<uintptr_t>(G)) % 16 == 0;
+  if (prec == P32 && Lsh >= 3 && Lsh <= 16 && aligned) {
     // CTAs of 64 threads for up to 8 pairs per site (8 or 16 sites; measured 108.2 us against 109.5 us
     // with 128 threads at 16^4 x 16, the same warps per SM and a finer last wave), 128 above
 #define FR(L_, T_)                                                                                       \

@@ -7,6 +7,8 @@ and the integer precision conversions bit for bit.
 Tolerances as in test_gpu_parity: FP64 1e-12, FP32 1e-5 (force 2e-5), 16-bit storage one output
 rounding per launch (2^-11, 2^-8) with the margin used there.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -297,4 +299,24 @@ def test_ragged_ends_and_short_warps(dwf, oracle_lib, monkeypatch, dims, Ls, spc
         r = oracle_lib.m(dims, Ls, M5, MASS, BC, U, op.unpack(x).cpu().numpy()) - psi
         assert np.linalg.norm(r) < 1e-8 * np.linalg.norm(psi)
     plain.close()
+    op.close()
+
+
+@pytest.mark.parametrize("Ls", [5, 8, 12, 18, 34])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_force_outputs_between_16_byte_boundaries(dwf, Ls, prec):
+    """F and G at odd multiples of 8 bytes: the same numbers, to FP32 rounding of a sum in another order."""
+    dims = (4, 2, 2, 4)
+    op = dwf.GridDWF(dims, Ls, M5, MASS, bc=BC)
+    op.set_gauge(dev(synth.random_gauge(dims, seed=781)))
+    f = op.pack(dev(synth.random_spinor(dims, Ls, seed=782)), prec, dwf.FULL)
+    chi = op.m(f)
+    _, F, G = op.force(f)
+    out = torch.zeros(2, F.numel() * 2 + 2, dtype=torch.float64, device="cuda")
+    at = [ctypes.c_void_p(row.data_ptr() + 8) for row in out]
+    op._call("grid_dwf_force_contract", prec, dwf._ptr(f), dwf._ptr(chi), *at)
+    for row, want in zip(out.cpu().numpy(), (F, G)):
+        assert row[0] == 0 and row[-1] == 0
+        got = row[1:-1].view(np.complex128).reshape(want.shape)
+        assert rel(got, want.cpu().numpy()) < (1e-14 if prec == 0 else 2e-5)
     op.close()
