@@ -144,88 +144,6 @@ __device__ __forceinline__ void project(int mu, const R* psi, R* h) {
 #undef PI
 }
 
-template <typename R>
-__device__ __forceinline__ R fma_r(R a, R b, R c);
-template <>
-__device__ __forceinline__ float fma_r<float>(float a, float b, float c) {
-  return fmaf(a, b, c);
-}
-template <>
-__device__ __forceinline__ double fma_r<double>(double a, double b, double c) {
-  return fma(a, b, c);
-}
-
-// acc += c * reconstruct(uh): upper spins take uh, lower spins the matching multiple of it.
-// c carries the boundary phase and any overall scale, so each term is one FMA.
-template <int SIG, typename R>
-__device__ __forceinline__ void accumulate(int mu, const R* uh, R c, R* acc) {
-  const R cs = SIG * c;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const R a0r = uh[(0 * 3 + k) * 2], a0i = uh[(0 * 3 + k) * 2 + 1];
-    const R a1r = uh[(1 * 3 + k) * 2], a1i = uh[(1 * 3 + k) * 2 + 1];
-    R* s0 = acc + (0 * 3 + k) * 2;
-    R* s1 = acc + (1 * 3 + k) * 2;
-    R* s2 = acc + (2 * 3 + k) * 2;
-    R* s3 = acc + (3 * 3 + k) * 2;
-    s0[0] = fma_r(c, a0r, s0[0]);
-    s0[1] = fma_r(c, a0i, s0[1]);
-    s1[0] = fma_r(c, a1r, s1[0]);
-    s1[1] = fma_r(c, a1i, s1[1]);
-    if (mu == 0) {  // spin2 += SIG i uh1, spin3 += SIG i uh0
-      s2[0] = fma_r(-cs, a1i, s2[0]);
-      s2[1] = fma_r(cs, a1r, s2[1]);
-      s3[0] = fma_r(-cs, a0i, s3[0]);
-      s3[1] = fma_r(cs, a0r, s3[1]);
-    } else if (mu == 1) {  // spin2 += SIG uh1, spin3 -= SIG uh0
-      s2[0] = fma_r(cs, a1r, s2[0]);
-      s2[1] = fma_r(cs, a1i, s2[1]);
-      s3[0] = fma_r(-cs, a0r, s3[0]);
-      s3[1] = fma_r(-cs, a0i, s3[1]);
-    } else if (mu == 2) {  // spin2 += SIG i uh0, spin3 -= SIG i uh1
-      s2[0] = fma_r(-cs, a0i, s2[0]);
-      s2[1] = fma_r(cs, a0r, s2[1]);
-      s3[0] = fma_r(cs, a1i, s3[0]);
-      s3[1] = fma_r(-cs, a1r, s3[1]);
-    } else {  // spin2 += SIG uh0, spin3 += SIG uh1
-      s2[0] = fma_r(cs, a0r, s2[0]);
-      s2[1] = fma_r(cs, a0i, s2[1]);
-      s3[0] = fma_r(cs, a1r, s3[0]);
-      s3[1] = fma_r(cs, a1i, s3[1]);
-    }
-  }
-}
-
-// o = U h (DAGGER = false) or U^+ h, for both spins of the half spinor; u row-major 3x3 complex.
-// Written as explicit FMA chains: 12 instructions per complex output.
-template <bool DAGGER, typename R>
-__device__ __forceinline__ void su3_mul(const R* u, const R* h, R* o) {
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      R re, im;
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int e = DAGGER ? (b * 3 + a) : (a * 3 + b);
-        const R ur = u[e * 2];
-        const R ui = DAGGER ? -u[e * 2 + 1] : u[e * 2 + 1];
-        const R hr = h[(sp * 3 + b) * 2], hi = h[(sp * 3 + b) * 2 + 1];
-        if (b == 0) {
-          re = ur * hr;
-          im = ur * hi;
-        } else {
-          re = fma_r(ur, hr, re);
-          im = fma_r(ur, hi, im);
-        }
-        re = fma_r(-ui, hi, re);
-        im = fma_r(ui, hr, im);
-      }
-      o[(sp * 3 + a) * 2] = re;
-      o[(sp * 3 + a) * 2 + 1] = im;
-    }
-}
-
 // Third row of an SU(3) matrix from its first two: row2 = conj(row0 x row1).
 template <typename R>
 __device__ __forceinline__ void reconstruct_row2(R* u) {
@@ -575,14 +493,6 @@ __device__ __forceinline__ void load_lane64(const char* blk, int s, int Lsh_rt, 
     const double* p = reinterpret_cast<const double*>(b + k * chunk_stride(Lsh));
     v[k] = GLOBAL ? __ldg(p) : *p;
   }
-}
-
-template <int LSH>
-__device__ __forceinline__ void store_lane64(char* blk, int s, int Lsh_rt, const double* v) {
-  const int Lsh = LSH > 0 ? LSH : Lsh_rt;
-  char* b = blk + (size_t)s * 8;
-#pragma unroll
-  for (int k = 0; k < 24; ++k) *reinterpret_cast<double*>(b + k * chunk_stride(Lsh)) = v[k];
 }
 
 // Packed precisions: reals r0 .. r0 + 11 (r0 = 0: the upper, P+ spins; 12: the lower) of slice s,
@@ -1042,7 +952,6 @@ inline int dhop_threads_per_site(int prec, int Ls) { return prec == P64 ? ls_pad
 // Float-float kernel: Ls values with a compile-time specialisation; any other Ls runs the generic kernel
 // (LSC = 0).
 #define DWF_LS_SPECIALISATIONS(M) M(8) M(12) M(16)
-inline bool dhop_ls_specialised(int Ls) { return Ls == 8 || Ls == 12 || Ls == 16; }
 
 // C12 selects the stored link format; LSHC = Ls / 2 for the extents compiled in, 0 for any; EK the epilogue kind.
 template <int P, bool DAG, bool C12, int LSHC, int EK>

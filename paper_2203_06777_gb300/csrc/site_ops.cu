@@ -914,32 +914,6 @@ cudaError_t launch_accum_zero(int py, void* x, void* y, long nsites, int Ls, con
   }
   return cudaGetLastError();
 }
-
-template <int P>
-__global__ void k_axpby(double a, const void* x, double b, void* y, UnitMap um) {
-  using R = RT<P>;
-  for (long u = blockIdx.x * (long)blockDim.x + threadIdx.x; u < um.units; u += (long)gridDim.x * blockDim.x) {
-    R xv[16], yv[16];
-    ld_unit<P, true>(x, um, u, xv);
-    ld_unit<P, true>(y, um, u, yv);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) yv[j] = R(a) * xv[j] + R(b) * yv[j];
-    st_unit<P>(y, um, u, yv);
-  }
-}
-
-cudaError_t launch_axpby(int p, double a, const void* x, double b, void* y, long nsites, int Ls, cudaStream_t st) {
-  const UnitMap um = unit_map(nsites, Ls);
-  const int blocks = grid_for(um.units, 256);
-  switch (p) {
-    case P64: k_axpby<P64><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
-    case P32: k_axpby<P32><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
-    case P16: k_axpby<P16><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
-    default: k_axpby<PB16><<<blocks, 256, 0, st>>>(a, x, b, y, um); break;
-  }
-  return cudaGetLastError();
-}
-
 }  // namespace gdwf
 
 // ---------------------------------------------------------------- reduction without allocation

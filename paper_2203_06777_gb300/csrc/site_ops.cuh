@@ -176,7 +176,5 @@ cudaError_t launch_residual64(const void* b, const void* Ax, void* r, long nsite
                               const Final& f, cudaStream_t st);
 // x (FP64) += c * y (precision py), then y = 0, with c = *c_dev.
 cudaError_t launch_accum_zero(int py, void* x, void* y, long nsites, int Ls, const double* c_dev, cudaStream_t st);
-// y = a x + b y elementwise in precision p (a, b host scalars).
-cudaError_t launch_axpby(int p, double a, const void* x, double b, void* y, long nsites, int Ls, cudaStream_t st);
 
 }  // namespace gdwf
