@@ -444,7 +444,7 @@ def run_force(dwf, torch, spec, reps=20):
     ms64ff = e0.elapsed_time(e1) / reps
     op.close()
     return {"workload": "dwf_16x16x16x16_ls16_haar", "ms_per_force": round(ms, 4), "reps": reps,
-            "precision": "fp32 fields, fp64 accumulation across blocks of 8 slice pairs",
+            "precision": "fp32 fields, fp32 products and slice sums, fp64 F and G",
             "ms_per_force_fp64": round(ms64, 4), "ms_per_force_fp64_float_float": round(ms64ff, 4),
             "includes": "M psi with |M psi|^2 summed in the same launch (Dhop with the fused Mooee term and norm, both halves), force and ambient-gradient kernel"}
 

@@ -251,8 +251,13 @@ int hop_full_cta_sites(const grid_dwf_t* h, int prec) {
 
 // Where that does not divide the half lattice's N sites, the ragged end needs a second launch, which
 // the next one waits for (about 4 us): then the divisor of N that fills its warps best is taken
-// instead, unless the lanes that it leaves idle cost more. Mpc^+ Mpc at 14x10x6x18 x 10 (7560 =
-// 302 x 25 + 10 = 315 x 24 sites): 82 -> 64 us (generic Ls kernel).
+// instead, unless the lanes that it leaves idle cost more. Divisor and second launch, full hop / Mpc in
+// us, at the idle lanes' estimated cost (below):
+//   14^4 x 12, 1.2 us: FP32 33 / 40 and 41 / 53, FP16 24 / 31 and 27 / 41, BF16 25 / 32 and 29 / 43;
+//   18^4 x 12, 4.1 us: FP32 82 / 107 and 84 / 117, FP16 67 / 82 and 68 / 88, BF16 69 / 85 and 70 / 92;
+//   26^4 x 6, 10.7 us: FP32 223 / 286 and 222 / 303, FP16 170 / 217 and 159 / 226, BF16 172 / 219 and 158 / 226;
+//   22^4 x 12, 14.6 us: FP32 181 / 219 and 173 / 223, FP16 153 / 178 and 137 / 168, BF16 162 / 188 and 145 / 176.
+// So the divisor wins up to the line at 4 us and a little beyond, and by less as the cost grows.
 int hop_sites_per_cta(const grid_dwf_t* h, int prec) {
   const int N = h->g.N4h, full = hop_full_cta_sites(h, prec);
   if (prec == GRID_DWF_FP64 || N % full == 0 || full == h->spc) return full;
@@ -490,7 +495,7 @@ int grid_dwf_create(const int dims[4], int Ls, double M5, double mass, const int
     if (dims[m] < 2 || dims[m] % 2) return GRID_DWF_ERR_INVALID_ARG;
     V *= dims[m];
   }
-  if (Ls < 1 || Ls > 128) return GRID_DWF_ERR_INVALID_ARG;  // FP64: one thread per slice, 128 per CTA
+  if (Ls < 1 || Ls > 128) return GRID_DWF_ERR_INVALID_ARG;  // a CTA holds a site: at most 256 threads, two per slice (FP64)
   if ((V / 2) * 8 >= (1L << 31)) return GRID_DWF_ERR_INVALID_ARG;
   if (!std::isfinite(M5) || !std::isfinite(mass)) return GRID_DWF_ERR_INVALID_ARG;
   const int defbc[4] = {1, 1, 1, -1};

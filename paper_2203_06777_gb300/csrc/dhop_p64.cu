@@ -6,11 +6,11 @@
 // site and slice is 12 additions (projection), 72 FMAs (link times half spinor) and 24 FMAs
 // (accumulation), so a kernel in IEEE FP64 instructions spends 864 of them, 432 clocks, per 5D site
 // and measured 762 us per 16^4 x 16 half lattice (94% of that pipe, 5% of HBM). With the whole sum in
-// integers only the conversion of the 24 results stays on the FP64 pipe: 232 us per half lattice.
-// About 10,000 integer instructions per 5D site, spread over the shift/logic pipe (51% busy) and the
-// multiplier (55%), bound it now (53% of the issue slots; occupancies of 16 to 28 warps per SM run
-// within 7%). An earlier form with IEEE additions for the projection measured 235 us, and one thread
-// per slice (168 registers, 12 warps per SM) 280 us.
+// integers only the conversion of the 24 results stays on the FP64 pipe: 241 us per half lattice (233 us
+// before the check of small components, below). About 10,500 integer instructions per 5D site, on the
+// shift/logic pipe (55% busy) and the multiplier, bound it now (57% of the issue slots; occupancies of 16
+// to 28 warps per SM run within 7%). Without that check, IEEE additions for the projection measured 235 us,
+// and one thread per slice (168 registers, 12 warps per SM) 280 us.
 //
 // The arithmetic. The 24 reals of a neighbour's (site, slice) become a block of integers with one
 // binary exponent, that of the largest; so does every link, once, when the links are uploaded.
@@ -220,9 +220,10 @@ __device__ __forceinline__ long long fx_asr(long long v, int d) {
 // a + v with the sign of v flipped where m is -1 (m is 0 or -1)
 __device__ __forceinline__ long long fx_add_signed(long long a, long long v, long long m) { return a + (v ^ m) + (m & 1); }
 
-// 80 registers: six CTAs of 128 threads per SM. 16^4 x 16 Mpc^+ Mpc at 72 / 80 / 96 / 128 registers:
-// 1001 / 1016 / 1032 / 1070 us, 24^4 x 12: 4200 / 4146 / 4197 / 4330 us; the next hop's loads issued
-// before this hop's products (24 more registers) 1080-1110 us.
+// 80 registers: six CTAs of 128 threads per SM. 16^4 x 16 Mpc^+ Mpc at 72 / 80 / 88 / 96 registers:
+// 1049 / 1057 / 1068 / 1049 us; without the check of small components at 72 / 80 / 96 / 128 1001 / 1016 /
+// 1032 / 1070 us, 24^4 x 12 4200 / 4146 / 4197 / 4330 us, and with the next hop's loads issued before this
+// hop's products (24 more registers) 1080-1110 us.
 template <int LSC>
 __global__ void __maxnreg__(80) dhop_kernel_fx(const __grid_constant__ DhopArgs a, bool dag, bool c12) {
   constexpr int LSHC = LSC > 0 ? ls_half(LSC) : 0;

@@ -18,9 +18,9 @@
 // threads form their slices' contributions to B1 and B2 of the link U_mu(x) leaving their site
 // (the own spinors and the two x + mu neighbours, the same loads as one Dhop hop), the CTA sums
 // them over the site's slices through shared memory, and the link algebra is spread over the
-// CTA's threads (one 3x3 entry each). FP32 fields: the products are summed in FP32 over blocks of
-// at most 8 slice pairs and the block sums in FP64, and the link algebra (U B1, B2 U^+, the
-// traceless anti-Hermitian projection) runs in FP32 on those sums: GB300's FP64 pipe is 1/64 of
+// CTA's threads (one 3x3 entry each). FP32 fields: the products are summed in FP32 over up to 16 slice
+// pairs (k_force_reg) or over blocks of 8 pairs whose sums are added in FP64 (k_force), and the link
+// algebra (U B1, B2 U^+, the traceless anti-Hermitian projection) runs in FP32 on those sums: GB300's FP64 pipe is 1/64 of
 // its FP32 pipe, and FP64 algebra made the kernel 5x slower for an answer whose error is set by
 // the FP32 fields and block sums anyway. FP64 fields: k_force_fx below. F and G are written
 // in the canonical FP64 layout [t][z][y][x][mu][3][3].
@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(128) k_force(const Geom g, const char* psi, co
 //     and adds its partner's copy of that half), after which lane q holds entries
 //     q * NPAD / LSH .. of the site's sum; those go to shared memory.
 //   - The link algebra of the site's four links (36 entries) is spread over the same lanes.
-// Rounding: the products of a slice pair and the sums over at most 16 pairs are FP32, as in the
-// general kernel (which flushes to FP64 after 8 pairs; here 16 pairs at most are summed in FP32).
+// Rounding: the products of a slice pair and the sums over at most 16 pairs are FP32, pairwise. The general
+// kernel adds 8 pairs one after the other in FP32, and two such blocks in FP64 before one rounding, which
+// is the FP32 sum of the two; so this order rounds less often. 2-norm errors with 9 to 15 pairs, in 1e-7:
+// F 1.29-1.35 here and 1.36-1.40 there, G 0.64-0.71 and 0.68-0.76.
 template <int LG, int THREADS>
 struct ForceRegGeom {
   static constexpr int SPC = THREADS / LG;               // sites per CTA
@@ -405,7 +407,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_force_reg(const Geom
 // largest slice's exponent while they are added over the site's slices, and rounded to FP64 once. The
 // link algebra of all four directions follows at the end, in FP64, 36 entries per site (direction by
 // direction, with 36 of 128 threads at work between barriers: force call at 16^4 x 16 1612 us; with
-// FP64 products 2520 us; now 1288 us, of which M psi is 470 us). Integer instructions and the barriers
+// FP64 products 2520 us; now 1311 us, of which M psi is 480 us). Integer instructions and the barriers
 // around the slice sums bound it now.
 // IEEE instructions instead: for a block of sites with a magnitude outside the integer range, all its
 // slices (force_products_ieee); and for an entry of B1 or B2 whose slices' |re| + |im| sum to less than an

@@ -378,8 +378,8 @@ cudaError_t launch_convert(int psrc, int pdst, const void* src, void* dst, long 
 // of the chirality coupled to s - 1 is, with S_s = sum_{1 <= k <= s} b_k d^-(s-k+1),
 //   y_0 = (b_0 - m S_{Ls-1}) / (d + m d^-(Ls-1)),  y_s = S_s + d^-s y_0,
 // S by a scan over the lanes; y so formed on the pair before feeds the recurrence y_s = (b_s + y_{s-1}) / d
-// over a pair's own slices (its rounding damped by 1 / d). The other chirality is the mirror image in s. Bound by memory in FP32 and 16 bits: inverse at 24^4 x 12 full, FP32, 192 -> 129 us (5.9 TB/s),
-// forward half field 84 -> 59 us. The shared-memory
+// over a pair's own slices (its rounding damped by 1 / d). The other chirality is the mirror image in s. Bound by memory in FP32 and 16 bits: inverse at 24^4 x 12 full, FP32, 192 -> 131 us
+// (5.8 TB/s), forward half field 84 -> 59 us. The shared-memory
 // kernel below, which served every case before, stages the field between barriers and runs each
 // line's two sweeps serially. Without the compile-time number of scan steps: 174 us.
 struct InvPowers {

@@ -1,5 +1,6 @@
-"""Every fifth-dimension extent around the limits of the kernels' dispatch, on lattices whose CTAs do not
-come out even, against the FP64 oracle: hopping term and Schur operator (even Ls to 24 and 32 are
+"""Every fifth-dimension extent around the limits of the kernels' dispatch, on lattices that full
+CTAs do not divide (the launches then take a divisor, or the caller's count and a second launch for the
+end), against the FP64 oracle: hopping term and Schur operator (even Ls to 24 and 32 are
 compiled in, the rest is generic), the fifth-dimension term (warp shuffles to 32 slice pairs, shared
 memory above and for the FP64 inverse), the force (3 to 16 pairs in registers; FP64 in block integers),
 and the integer precision conversions bit for bit.

@@ -4,7 +4,8 @@ launch would overwrite the guard), and its output is finite.
 
 Each output is the middle of a larger byte buffer whose guards hold a fixed byte pattern; after
 the call the pattern must be intact. Lattices include an odd Ls (a zero pad slice), a half
-lattice that is not a multiple of the sites per CTA (the extra tail launch) and the largest Ls.
+lattice that is not a multiple of a full CTA's sites and the largest Ls; test_gpu_extents sets the sites
+per CTA so that the lattice's end takes a launch of its own.
 """
 import ctypes
 

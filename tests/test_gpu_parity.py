@@ -335,8 +335,8 @@ def test_mixed_cg_stopped_by_maxiter(dwf, oracle_lib, mode):
 # ---------------------------------------------------------------- force
 
 
-# (4, 4, 4, 6) x 10: 192 sites per parity in CTAs of 25, so the FP32 M launch that also sums the
-# action has end CTAs (one per half) beside its full ones.
+# (4, 4, 4, 6) x 10: 192 sites per parity, which full CTAs of 25 do not divide (the FP32 M launch that
+# also sums the action takes CTAs of 24).
 @pytest.mark.parametrize("dims,Ls", [((4, 4, 4, 4), 4), ((2, 4, 2, 6), 3), ((4, 2, 4, 2), 16), ((4, 4, 4, 6), 10)])
 @pytest.mark.parametrize("prec", [0, 1])
 def test_force_parity(dwf, oracle_lib, dims, Ls, prec):
@@ -592,7 +592,7 @@ def test_force_8x8x8x8_ls8_fd_and_oracle(dwf, oracle_lib):
 
 # ---------------------------------------------------------------- random-shape sweep
 # Seeded random lattice shapes (each extent 2, 4 or 6; Ls in 1..16) against the oracle: ragged
-# half lattices, odd Ls (pad slice), tail launches and every Ls specialisation and the generic
+# half lattices, odd Ls (pad slice) and every Ls specialisation and the generic
 # kernel, for the hopping term (both signs) and the full M.
 
 def _random_shapes(n=12, seed=2203):
