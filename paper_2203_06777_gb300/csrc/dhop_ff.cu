@@ -6,7 +6,7 @@
 // HBM needs for its bytes. A float-float operation costs between 2 and 12 FP32 instructions, so the
 // operator runs on the wide FP32 pipe instead: 261 us per 16^4 x 16 half lattice, 762 us in FP64
 // instructions. The default FP64 kernel (dhop_p64.cu) leaves the FP64 pipe too, for 64-bit integers:
-// 233 us at full FP64 precision, so the plain hop no longer gains from this one. The format is Dekker's double-length arithmetic ("A floating-point technique
+// 241 us at full FP64 precision, so the plain hop no longer gains from this one. The format is Dekker's double-length arithmetic ("A floating-point technique
 // for extending the available precision", Numer. Math. 18, 1971): a sum is formed with Knuth's
 // error-free TwoSum, a product with the FMA-based TwoProduct (the rounding error of a*b is
 // fma(a, b, -a*b) exactly). A value carries about 47 significant bits (2^-47 ~ 7e-15 relative),
