@@ -85,7 +85,8 @@ typedef struct {
  * dims[4] = {Lx, Ly, Lz, Lt}, each even and >= 2, Lx*Ly*Lz*Lt/2 < 2^31 / 8; 1 <= Ls <= 128;
  * M5, mass finite, and Mooee invertible for them; bc[4] each +1 (periodic) or -1
  * (antiperiodic), NULL meaning {+1, +1, +1, -1}; compress12 != 0 stores links as two rows (the
- * third rebuilt as the conjugated cross product, exact for SU(3) links); stream is a
+ * third rebuilt as the conjugated cross product, exact for SU(3) links; the native FP64 hop holds all
+ * three as integers, 160 bytes per link); stream is a
  * cudaStream_t (NULL = legacy default stream). Uses the current CUDA device. On success *out
  * owns device memory for the links and workspaces, freed by grid_dwf_destroy.
  * Tuning read from the environment at create (the operators' results are the same bit for bit
