@@ -116,8 +116,9 @@ int grid_dwf_set_stream(grid_dwf_t* h, void* stream);
  * 64-bit integer blocks: a neighbour's 24 reals of one slice, and a link's 18, share the exponent of
  * the largest (57 and 58 bits below it are kept), the product of two low digits is dropped, and one
  * rounding per hop follows. Errors are below those of IEEE arithmetic relative to the largest real of the
- * (site, slice)'s neighbours, and at most 2^-42 (2^-49 rms) of the sum of magnitudes of any complex
- * component's own terms. A (site, slice) whose components are too unequal for that, or a magnitude
+ * (site, slice)'s neighbours, and at most 2^-42 of the sum of magnitudes of any complex component's own
+ * terms (on Gaussian fields and propagators 2^-56 to 2^-54 rms and 2^-49.6 at most; IEEE 2^-54.5 to 2^-54
+ * and 2^-51). A (site, slice) whose components are too unequal for that, or a magnitude
  * outside 2^-400 .. 2^400 (infinities, NaN and subnormals included), is computed in IEEE double. The
  * FP64 force forms its outer products and their sums over the slices in the same way, and in IEEE double
  * any entry far below the largest product of its site's slices. The rest of the operators and of the

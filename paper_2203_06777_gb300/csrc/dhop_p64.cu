@@ -32,9 +32,10 @@
 // z and t (9 of about 640 instructions per thread and hop; Mpc^+ Mpc at 16^4 x 16 1016 -> 1050 us), and a
 // (site, slice) with a complex component for which neither sum reaches an eighth of the smallest product of
 // two blocks' largest reals (2^53 accumulator units) is computed with IEEE FP64 instructions. The errors
-// above are at most 92 units per real over the eight hops (1 unit rms), so a component's error is at most
-// 2^-42 (2^-49 rms) of the sum of its terms' magnitudes, at the limit; typically they sum to 8 x 2^53
-// units. Gaussian fields stay above the limit (none of 4e5 simulated sites below), propagators on random
+// above are at most 92 units per real over the eight hops (about 1 unit rms), so a component's error is at
+// most 2^-42 of the sum of its terms' magnitudes; measured against quadruple precision (8^4 x 8, Gaussian
+// fields, point and wall propagators, random and smooth links) rms 0.12-0.37 x 2^-53, 99.9% below 2.1 x 2^-53,
+// all below 10 x 2^-53; in IEEE instructions 0.34-0.45, 2.0 and 3.7. Gaussian fields stay above the limit (none of 4e5 simulated sites below), propagators on random
 // and on smooth links nearly everywhere (3e-5 of the sites of an 8^4 x 8 point source's); a limit of 2^53
 // would send 17-43% of the latter to IEEE instructions. Components all of whose terms are 0 (a source's
 // empty spins and colours) come out exactly 0 either way and stay.
